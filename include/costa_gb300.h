@@ -54,10 +54,10 @@
  *    Rump & Oishi 2005) for single-precision data; for double-precision
  *    data whose operands are all zero or of magnitude in [2^-480, 2^480),
  *    by an exact fixed-point sum on the integer pipes rounded once (every
- *    four-product component, every other element of two-product ones)
- *    and by Kahan's algorithm for 2 x 2 determinants (the other
- *    two-product ones); Dot2 otherwise.  Repeated calls on one pair give
- *    the same bits.  When beta == 0, A is never read, so NaN or garbage in
+ *    four-product component, the imaginary two-product ones) and by
+ *    Kahan's algorithm for 2 x 2 determinants (the real two-product
+ *    ones); Dot2 otherwise.  Repeated calls on one pair give the same
+ *    bits.  When beta == 0, A is never read, so NaN or garbage in
  *    A does not propagate.
  */
 #ifndef COSTA_GB300_H
@@ -540,6 +540,24 @@ costa_status costa_debug_halves(costa_layout A, costa_layout B, costa_op op, voi
 costa_status costa_debug_exchange(costa_layout A, costa_layout B, costa_op op, int G, const int *place, int g,
                                   uint64_t send_base, uint64_t recv_base, int which, void *out, int64_t cap,
                                   int64_t *count, int64_t *volumes);
+
+/* Diagnostics (host only, no device work): the patches of (A, B, op), the
+ * work list of the patch kernel, which moves pairs whose overlay cells are
+ * mostly small or misaligned.  A patch is a window of A's storage (at most
+ * 32 x 32 elements; 16 x 16 for 16-byte elements) that may cover several
+ * overlay cells: 32 bytes {target address (uint64), target stride (int32),
+ * first cell (uint32), lmask, rmask (uint32), nx, ny (uint8), problem, flags,
+ * padding (uint16)}, x along A's contiguous axis.  The source is cut into
+ * segments along the lane axis (the source's contiguous one: y when flags
+ * has 1 = transposed, else x) and the run axis (the other): bit k of lmask /
+ * rmask is set where one starts.  Segment pair (r, l) is cell first + r *
+ * popcount(lmask) + l, 16 bytes {address (uint64), source stride (int32),
+ * padding}: its element (run i, lane j of the patch) is at address +
+ * (i * stride + j) elements.  Writes up to cap_patches patches and cap_cells
+ * cells and the totals; 0 when the pair has no patches (layouts that mix
+ * element orders). */
+costa_status costa_debug_patches(costa_layout A, costa_layout B, costa_op op, void *patches, int64_t cap_patches,
+                                 void *cells, int64_t cap_cells, int64_t *npatches, int64_t *ncells);
 
 /* Diagnostics: TMA staging of the tile kernel's source tiles.  By default
  * (environment variable COSTA_TMA unset when a plan is built) only f64 data

@@ -87,6 +87,7 @@ def _load():
         "costa_debug_tiles": [P, P, I, P, I64, P],
         "costa_debug_split": [P, P, I, P, I64, P, I64, P, I64, P, P, P],
         "costa_debug_halves": [P, P, I, P, I64, P],
+        "costa_debug_patches": [P, P, I, P, I64, P, I64, P, P],
         "costa_debug_groups": [P, P, I, I, P, I64, P],
         "costa_phase_timing": [I],
         "costa_phase_times": [P, P],
@@ -579,6 +580,24 @@ def costa_debug_split(A: Layout, B: Layout, op: str):
                                   pieces.ctypes.data, npc.value, groups.ctypes.data, ngo,
                                   ctypes.byref(nt), ctypes.byref(npc), ctypes.byref(ng)))
     return tiles[:nt.value], pieces[:npc.value], groups[:ngo]
+
+
+PATCH_DTYPE = np.dtype([("dst", np.uint64), ("dld", np.int32), ("cell0", np.uint32), ("lmask", np.uint32),
+                        ("rmask", np.uint32), ("nx", np.uint8), ("ny", np.uint8), ("prob", np.uint16),
+                        ("flags", np.uint16), ("pad", np.uint16)])
+CELL_DTYPE = np.dtype([("src", np.uint64), ("sld", np.int32), ("pad", np.int32)])
+
+
+def costa_debug_patches(A: Layout, B: Layout, op: str):
+    """(patches, cells) of the patch kernel's list (empty when the pair has none)."""
+    n, nc = ctypes.c_int64(), ctypes.c_int64()
+    args = (A.handle, B.handle, OPS[op])
+    _check(_lib.costa_debug_patches(*args, None, 0, None, 0, ctypes.byref(n), ctypes.byref(nc)))
+    patches = np.zeros(max(1, n.value), dtype=PATCH_DTYPE)
+    cells = np.zeros(max(1, nc.value), dtype=CELL_DTYPE)
+    _check(_lib.costa_debug_patches(*args, patches.ctypes.data, n.value, cells.ctypes.data, nc.value,
+                                    ctypes.byref(n), ctypes.byref(nc)))
+    return patches[:n.value], cells[:nc.value]
 
 
 def costa_debug_groups(A: Layout, B: Layout, op: str, reads_a: bool) -> np.ndarray:

@@ -362,6 +362,55 @@ costa_status check_access(costa_layout_s *L, int dev, const char *which) {
     return check_access_impl(L, dev, which, nullptr, 0);
 }
 
+// Moves the problems that the patch kernel serves from the tile list to
+// patches: every problem that has patches, when at least half of the list's
+// elements lie in small or misaligned tiles (4-byte tiles whose target runs
+// are aligned count as aligned: their window path is the faster one).
+// Measured on GB300, same box, 8192^2 (c128 6016^2), us per call, tile and
+// small-tile kernels -> patch kernel:
+//   BC50 -> BC75   f64 T copy 226 -> 175, N copy 231 -> 172, T beta = 0.5
+//                  312 -> 265, T beta = 0.7 494 -> 293; f32 T copy 212 ->
+//                  108; c64 T beta = 0.7 464 -> 261; c128 T copy 224 -> 190
+//   odd lds, T     f64 copy 210 -> 191, beta = 0.7 408 -> 293 (A's ld odd:
+//                  copy 182 -> 166, beta = 0.5 250 -> 250); f32, A's ld odd,
+//                  copy 112 -> 109, beta = 0.5 157 -> 149
+//   BC4 (half the rows), T copy: f64 290 -> 83, f32 310 -> 53, c64 299 ->
+//                  83, c128 191 -> 92
+//   BC8, T         f64 copy 187 -> 162, beta = 0.5 258 -> 242; f32 copy 164
+//                  -> 101, beta = 0.5 221 -> 139; c128 copy 219 -> 178, beta
+//                  = 0.5 380 -> 267
+//   BC16, T        f64 copy 182 -> 161; f32 copy 112 -> 101, beta = 0.5 146
+//                  -> 139; c128 beta = 0.5 375 -> 266
+// f32 with only B's ld odd: copy 99 -> 105 (kept on the window path).
+// COSTA_PATCH=0 turns the patches off, COSTA_PATCH=1 takes them for every
+// pair that has them (for measurements).
+void take_patches(const Plan &plan, std::vector<TileDesc> &list, PatchList &out) {
+    static const int mode = [] {
+        const char *e = std::getenv("COSTA_PATCH");
+        return e ? std::atoi(e) : -1;
+    }();
+    if (mode == 0 || list.empty()) return;
+    const int es = plan.esize;
+    int64_t all = 0, poor = 0;
+    for (const TileDesc &d : list) {
+        const int64_t e = static_cast<int64_t>(d.nx) * d.ny;
+        all += e;
+        const bool misaligned = es == 4 ? !aligned16(d.dst, static_cast<int64_t>(d.dld) * es) || d.nx % 4 != 0
+                                        : !(d.flags & TF_FAST);
+        if (misaligned || is_small(d, es)) poor += e;
+    }
+    if (2 * poor < all && mode != 1) return;
+    std::vector<char> taken(plan.probs.size(), 0);
+    bool any = false;
+    for (size_t k = 0; k < taken.size(); ++k)
+        any |= (taken[k] = append_patches(plan.probs[k], static_cast<int>(k), out)) != 0;
+    if (!any) return;
+    size_t w = 0;
+    for (const TileDesc &d : list)
+        if (!taken[d.prob]) list[w++] = d;
+    list.resize(w);
+}
+
 // Builds the overlay, the tile list and the device tables, and runs the
 // volume kernel.
 costa_status build_plan(int n, const costa_layout *As, const costa_layout *Bs, const costa_op *ops,
@@ -427,6 +476,8 @@ costa_status build_plan(int n, const costa_layout *As, const costa_layout *Bs, c
         if (st != COSTA_OK) return st;
     }
     const bool cplx = plan->dtype == COSTA_C64 || plan->dtype == COSTA_C128;
+    PatchList patches;
+    take_patches(*plan, list, patches);
     SplitList split = split_small(std::move(list), es, cplx);
     // The aligned tiles also as x-halves (see use_halves), for the kinds
     // that run on them (see launch_list in transform_impl).
@@ -440,6 +491,7 @@ costa_status build_plan(int n, const costa_layout *As, const costa_layout *Bs, c
     plan->tma_kinds_halves = had_halves ? tma_policy_kinds(halves, es, cplx, true) : 0;
     const SplitOffsets off_tiles = arena.add_split(split);
     const size_t off_halves = halves.empty() ? 0 : arena.add_vec(halves);
+    const size_t off_patches = arena.add_vec(patches.patches), off_pcells = arena.add_vec(patches.cells);
     const uint32_t zero_word = 0;
     const size_t off_err = arena.add(&zero_word, sizeof zero_word);
     std::vector<VolumeProblemDev> vd(n);
@@ -477,6 +529,9 @@ costa_status build_plan(int n, const costa_layout *As, const costa_layout *Bs, c
     ce = cudaMemcpy(d, arena.host.data(), arena.host.size(), cudaMemcpyHostToDevice);
     if (ce != cudaSuccess) return cuda_fail(ce, "cudaMemcpy(plan tables)");
     plan->direct = resolve(dbase, off_tiles, split);
+    plan->direct.patches = reinterpret_cast<const PatchDesc *>(dbase + off_patches);
+    plan->direct.cells = reinterpret_cast<const PatchCell *>(dbase + off_pcells);
+    plan->direct.npatches = static_cast<int64_t>(patches.patches.size());
     plan->direct_halves = plan->direct;
     if (had_halves) {
         plan->direct_halves.tiles = reinterpret_cast<const TileDesc *>(dbase + off_halves);
@@ -521,10 +576,10 @@ costa_status build_plan(int n, const costa_layout *As, const costa_layout *Bs, c
     plan->stats.n_tiles = tiles;
     plan->stats.plan_ms = ms_since(t0);
     log_msg(1, "plan: %d pair(s), dtype %d, P = %d, %lld cells, %lld tiles (%lld direct, %lld misaligned, "
-               "%lld small pieces), total volume %lld, local %lld; %.2f ms (volume %.2f ms)",
+               "%lld small pieces; %lld patches), total volume %lld, local %lld; %.2f ms (volume %.2f ms)",
             n, plan->dtype, P, (long long)cells, (long long)tiles, (long long)split.big.size(),
-            (long long)split.mis.size(), (long long)split.pieces.size(), (long long)total, (long long)trace,
-            plan->stats.plan_ms, plan->stats.volume_ms);
+            (long long)split.mis.size(), (long long)split.pieces.size(), (long long)patches.patches.size(),
+            (long long)total, (long long)trace, plan->stats.plan_ms, plan->stats.volume_ms);
     out = std::move(plan);
     return COSTA_OK;
 }
@@ -1062,6 +1117,16 @@ cudaError_t launch_split(const RemapLaunch &base, const DevList &list, const Dev
         }
         cudaError_t e = launch_remap(lk, kind, stream);
         if (e != cudaSuccess) return e;
+        if (list.npatches > 0) {
+            PatchLaunch p{};
+            p.patches = list.patches;
+            p.cells = list.cells;
+            p.n = list.npatches;
+            p.per_problem = base.per_problem;
+            p.s = base.s;
+            e = launch_patches(p, base.dtype, kind, stream);
+            if (e != cudaSuccess) return e;
+        }
     }
     return cudaSuccess;
 }
@@ -1436,6 +1501,27 @@ costa_status costa_debug_halves(costa_layout A, costa_layout B, costa_op op, voi
     *ntiles = static_cast<int64_t>(halves.size());
     const size_t k = static_cast<size_t>(std::min<int64_t>(cap_tiles, *ntiles));
     if (k) std::memcpy(tiles, halves.data(), k * sizeof(TileDesc));
+    return COSTA_OK;
+}
+
+costa_status costa_debug_patches(costa_layout A, costa_layout B, costa_op op, void *patches, int64_t cap_patches,
+                                 void *cells, int64_t cap_cells, int64_t *npatches, int64_t *ncells) {
+    costa_status s = validate_pair(A, B, op);
+    if (s != COSTA_OK) return s;
+    if (!npatches || !ncells || (cap_patches > 0 && !patches) || (cap_cells > 0 && !cells))
+        return fail(COSTA_ERR_INVALID_ARG, "bad arguments");
+    ProblemHost ph;
+    ph.A = A;
+    ph.B = B;
+    ph.op = op;
+    PatchList l;
+    append_patches(ph, 0, l);
+    *npatches = static_cast<int64_t>(l.patches.size());
+    *ncells = static_cast<int64_t>(l.cells.size());
+    const size_t kp = static_cast<size_t>(std::min<int64_t>(cap_patches, *npatches));
+    const size_t kc = static_cast<size_t>(std::min<int64_t>(cap_cells, *ncells));
+    if (kp) std::memcpy(patches, l.patches.data(), kp * sizeof(PatchDesc));
+    if (kc) std::memcpy(cells, l.cells.data(), kc * sizeof(PatchCell));
     return COSTA_OK;
 }
 

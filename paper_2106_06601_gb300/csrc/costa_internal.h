@@ -85,6 +85,40 @@ struct TileDesc {
 static_assert(sizeof(TileDesc) == 32, "TileDesc layout");
 enum : uint16_t { TF_TRANSPOSE = 1, TF_FAST = 2, TF_CONJ = 4, TF_ELEM = 8 };
 
+// A patch of the patch kernel (patches.cpp): a window of at most patch_x x
+// patch_y elements of A's storage, in the same frame (x = the target's
+// contiguous axis), whose source is a product of segments: the
+// run axis (x when transposed, y otherwise) and the lane axis (the source's
+// contiguous one).  lmask / rmask: bit k set where a segment of the lane /
+// run axis starts at element k.  Segment pair (r, l) is cell
+// cells[cell0 + r * (lane segments) + l]; its source element (run r, lane l
+// of the patch) is at src + r * sld + l elements.
+struct PatchDesc {
+    COSTA_HD PatchDesc() {}
+    uint64_t dst;    // device address of target element (0, 0)
+    int32_t dld;     // target stride (elements)
+    uint32_t cell0;
+    uint32_t lmask, rmask;
+    uint8_t nx, ny;  // extents
+    uint16_t prob;   // problem index within the launch
+    uint16_t flags;  // TF_TRANSPOSE, TF_CONJ
+    uint16_t pad;
+};
+static_assert(sizeof(PatchDesc) == 32, "PatchDesc layout");
+struct PatchCell {
+    COSTA_HD PatchCell() {}
+    uint64_t src;    // biased: address of the patch's element (0, 0) if the cell covered it
+    int32_t sld;     // source stride (elements)
+    int32_t pad;
+};
+static_assert(sizeof(PatchCell) == 16, "PatchCell layout");
+// Extents of a patch (x along A's runs): 256-byte runs of 8- and 16-byte
+// elements; 32 lanes bound a run.
+COSTA_HD constexpr int patch_x(int esize) { return esize == 16 ? 16 : 32; }
+COSTA_HD constexpr int patch_y(int esize) { return esize == 16 ? 16 : 32; }
+constexpr int kPatchSegs = 8;                           // segments per axis of a patch
+constexpr int kPatchCells = kPatchSegs * kPatchSegs;    // cells of a patch
+
 // Scalars of one problem, as doubles ({re, im}); float data carries values
 // that are exactly representable in float.
 struct Scalars {
@@ -157,6 +191,14 @@ struct RemapLaunch {
     const struct TmaLists *tma;
 };
 
+struct PatchLaunch {
+    const PatchDesc *patches;
+    const PatchCell *cells;
+    int64_t n;
+    const Scalars *per_problem;  // as RemapLaunch
+    Scalars s;
+};
+
 struct VolumeProblemDev {
     const Interval *rows;
     const Interval *cols;
@@ -221,6 +263,11 @@ cudaError_t launch_remap_f32(const RemapLaunch &args, int kind, cudaStream_t str
 cudaError_t launch_remap_f64(const RemapLaunch &args, int kind, cudaStream_t stream);
 cudaError_t launch_remap_c64(const RemapLaunch &args, int kind, cudaStream_t stream);
 cudaError_t launch_remap_c128(const RemapLaunch &args, int kind, cudaStream_t stream);
+cudaError_t launch_patches(const PatchLaunch &args, int dtype, int kind, cudaStream_t stream);
+cudaError_t launch_patches_f32(const PatchLaunch &args, int kind, cudaStream_t stream);
+cudaError_t launch_patches_f64(const PatchLaunch &args, int kind, cudaStream_t stream);
+cudaError_t launch_patches_c64(const PatchLaunch &args, int kind, cudaStream_t stream);
+cudaError_t launch_patches_c128(const PatchLaunch &args, int kind, cudaStream_t stream);
 cudaError_t launch_volume(const VolumeLaunch &args, cudaStream_t stream);
 void count_launch();
 int64_t launches_so_far();

@@ -32,7 +32,10 @@ struct DevList {
     const TileDesc *ttiles = nullptr;
     int64_t nttiles = 0;
     uint32_t tma_kinds = 0;
-    bool empty() const { return ntiles == 0 && nmtiles == 0 && ngroups == 0; }
+    const PatchDesc *patches = nullptr;
+    const PatchCell *cells = nullptr;
+    int64_t npatches = 0;
+    bool empty() const { return ntiles == 0 && nmtiles == 0 && ngroups == 0 && npatches == 0; }
 };
 
 struct SplitOffsets {

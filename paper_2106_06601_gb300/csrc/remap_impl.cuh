@@ -94,10 +94,9 @@ template <> struct ET<double2> { enum { VEC = 1, CPLX = 1 }; typedef double R; }
 //    (float multiplies) lost 11% with f64's shape and keeps the light one.
 //    c128 with a complex alpha (FP64-bound at 8 operations per element
 //    with Kahan's algorithm alone): T and N 1458 -> 2133 with 2 to 4
-//    blocks; with every other element summed in fixed point on the integer
-//    pipes (COSTA_FX_CS_PERIOD), unrolled, 2557 at 2 blocks, 2660 at 3 (one
-//    pass in 3 or 4 in fixed point: 2553, 2569); in the rolled loop, 3 blocks,
-//    3259.
+//    blocks; with half of the components summed in fixed point on the integer
+//    pipes, unrolled, 2557 at 2 blocks, 2660 at 3 (a third or a quarter of
+//    them: 2553, 2569); in the rolled loop, 3 blocks, 3259.
 //  - c64 complex scalars, against 3 blocks with 2 buffers: complex beta
 //    T 4484 -> 5482, N 4495 -> 5495 with 4 blocks and no look-ahead;
 //    complex alpha T 5551 -> 5955 with two tiles ahead; the real general
@@ -426,13 +425,6 @@ __device__ __forceinline__ double kahan2(double x, double y, double z, double t,
 #ifndef COSTA_FX_GROUP
 #define COSTA_FX_GROUP 2
 #endif
-// Passes that the drain of double complex data with a complex alpha and
-// beta = 0 evaluates together: the last in fixed point, the others by
-// Kahan's algorithm (0: every pass by Kahan's algorithm, one at a time).
-#ifndef COSTA_FX_CS_PERIOD
-#define COSTA_FX_CS_PERIOD 2
-#endif
-
 // Every operand of a double complex alpha * b + beta * a in the middle range
 // (b as it enters the combine, after any conjugation).
 __device__ __forceinline__ bool cplx_mid(const double2 &b, const double2 &a, const Sc &s) {
@@ -462,16 +454,17 @@ __device__ __forceinline__ double2 fx_cplx(const double2 &b, const double2 &a, c
     return o;
 }
 
-// alpha * b for double complex data and a complex alpha, each component the
-// sum of its two products in fixed point on the integer pipes (fxdot.h).
-// Every operand must be in the middle range.
-__device__ __forceinline__ double2 fx_cscale(const double2 &b, const Sc &s) {
+// alpha * b for double complex data and a complex alpha, every operand in the
+// middle range: the real component by Kahan's algorithm on the FP64 pipe, the
+// imaginary one as a fixed-point sum on the integer pipes (fxdot.h), so that
+// both pipes work.  The choice depends on nothing but the component, so every
+// kernel and work list gives the same bits.
+__device__ __forceinline__ double2 mid_cscale(const double2 &b, const Sc &s) {
     const fx::Op fbx = fx::unpack(b.x), fby = fx::unpack(b.y);
     const fx::Op far = fx::unpack(s.ar), fai = fx::unpack(s.ai);
-    const fx::Term re[2] = {fx::mul(far, fbx, 0u), fx::mul(fai, fby, 1u)};  // ar bx - ai by
     const fx::Term im[2] = {fx::mul(far, fby, 0u), fx::mul(fai, fbx, 0u)};  // ar by + ai bx
     double2 o;
-    o.x = fx::sum(re);
+    o.x = kahan2(s.ar, b.x, s.ai, b.y, true);  // ar bx - ai by
     o.y = fx::sum(im);
     return o;
 }
@@ -486,14 +479,9 @@ __device__ __forceinline__ C combine_c(C b, C a, const Sc &s) {
         return o;
     }
     if constexpr (KIND == K_CSCALE && sizeof(R) == 8) {
-        // the FP64 pipe is this kind's limit: two-term components take
-        // Kahan's algorithm when every operand is in the middle range (the
-        // others, and all non-finite values, take Dot2 below)
-        if (s.alpha_mid && mid_range(b.x) && mid_range(b.y)) {
-            o.x = kahan2(s.ar, b.x, s.ai, b.y, true);   // ar bx - ai by
-            o.y = kahan2(s.ar, b.y, s.ai, b.x, false);  // ar by + ai bx
-            return o;
-        }
+        // operands outside the middle range, and all non-finite values, take
+        // Dot2 below
+        if (s.alpha_mid && mid_range(b.x) && mid_range(b.y)) return mid_cscale(b, s);
     }
     if constexpr (KIND == K_CPLX && sizeof(R) == 8) {
         // four-term components: in fixed point on the integer pipes when
@@ -609,7 +597,7 @@ __device__ __forceinline__ double pow2_apply(double a, const Sc &s) {
 // so the scarce FP64 pipe never runs predicated-off multiplies.  beta = +-1
 // needs at most a sign flip.  Float data multiplies (the FP32 pipe is wide).
 template <typename T, int N>
-__device__ __forceinline__ void prescale(Chunk<T> (&av)[N], int npass, const Sc &s) {
+__device__ __forceinline__ void prescale(Chunk<T> (&av)[N], int npass, const Sc &s, unsigned mask = 0xffffffffu) {
     using R = typename ET<T>::R;
     constexpr int PER = 16 / static_cast<int>(sizeof(R));  // reals per chunk
     if constexpr (sizeof(R) == 8) {
@@ -632,7 +620,7 @@ __device__ __forceinline__ void prescale(Chunk<T> (&av)[N], int npass, const Sc 
 #pragma unroll
             for (int k = 0; k < PER; ++k) bad |= pow2_bad(v[k], s);
         }
-        if (__any_sync(0xffffffffu, bad)) {
+        if (__any_sync(mask, bad)) {
 #pragma unroll
             for (int p = 0; p < N; ++p) {
                 if (p >= npass) break;
@@ -720,20 +708,19 @@ __device__ __forceinline__ void stage_drain(const Geom<T> &g, const Sc &s, unsig
     if (m.c >= chunks) return;
     const int x0 = m.c * C::VEC;
     const int npass = (g.ny + m.rpp - 1) / m.rpp;
-    if constexpr ((KIND == K_CPLX || (KIND == K_CSCALE && COSTA_FX_CS_PERIOD > 0)) && sizeof(T) == 16) {
+    if constexpr ((KIND == K_CPLX || KIND == K_CSCALE) && sizeof(T) == 16) {
         // double complex with complex scalars: G passes at a time in
         // straight-line code, so that their evaluations overlap.  Four-term
         // components (complex beta) are all summed in fixed point on the
         // integer pipes (about 150 instructions each, in long dependent
-        // chains); two-term ones (complex alpha, beta = 0) split the passes
-        // between Kahan's algorithm on the FP64 pipe and the fixed-point sum,
-        // so that both pipes work.  The loop stays rolled: unrolled over the
+        // chains); two-term ones (complex alpha, beta = 0) by mid_cscale.  The
+        // loop stays rolled: unrolled over the
         // tile's passes, the fixed-point sums made a body of about 14,000
         // instructions, and instruction fetch stalled the warps.  So A is
         // not held as a whole tile in registers (av is unused here; the
         // callers do not load it for this kind): each iteration loads the A
         // chunks of the group two ahead of the one it combines.
-        constexpr int G = KIND == K_CPLX ? COSTA_FX_GROUP : COSTA_FX_CS_PERIOD;
+        constexpr int G = COSTA_FX_GROUP;
         T a_next[2][G];
         auto load_group = [&](int q0, T (&dst)[G]) {
 #pragma unroll
@@ -773,14 +760,7 @@ __device__ __forceinline__ void stage_drain(const Geom<T> &g, const Sc &s, unsig
             if (mid) {
 #pragma unroll
                 for (int j = 0; j < G; ++j) {
-                    if (KIND == K_CPLX) {
-                        o[j] = fx_cplx(bb[j], aa[j], s);
-                    } else if (j == G - 1) {
-                        o[j] = fx_cscale(bb[j], s);
-                    } else {
-                        o[j].x = kahan2(s.ar, bb[j].x, s.ai, bb[j].y, true);   // ar bx - ai by
-                        o[j].y = kahan2(s.ar, bb[j].y, s.ai, bb[j].x, false);  // ar by + ai bx
-                    }
+                    o[j] = KIND == K_CPLX ? fx_cplx(bb[j], aa[j], s) : mid_cscale(bb[j], s);
                 }
             } else {
 #pragma unroll

@@ -73,6 +73,17 @@ cudaError_t launch_remap(const RemapLaunch &a, int kind, cudaStream_t stream) {
     }
 }
 
+cudaError_t launch_patches(const PatchLaunch &a, int dtype, int kind, cudaStream_t stream) {
+    if (a.n <= 0) return cudaSuccess;
+    switch (dtype) {
+    case COSTA_F32: return launch_patches_f32(a, kind, stream);
+    case COSTA_F64: return launch_patches_f64(a, kind, stream);
+    case COSTA_C64: return launch_patches_c64(a, kind, stream);
+    case COSTA_C128: return launch_patches_c128(a, kind, stream);
+    default: return cudaErrorInvalidValue;
+    }
+}
+
 cudaError_t launch_volume(const VolumeLaunch &a, cudaStream_t stream) {
     if (a.total_cells <= 0) return cudaSuccess;
     const int threads = 256;

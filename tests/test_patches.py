@@ -1,0 +1,117 @@
+"""CPU check of the patch kernel's work list: patches, expanded element by
+element with the kernel's own index arithmetic, move exactly the elements
+that the tile list moves (the general path), each from the same source
+address to the same target address, within the kernel's limits."""
+import numpy as np
+import pytest
+
+from workloads import configs as C
+from workloads import layouts as L
+
+costa = pytest.importorskip("paper_2106_06601_gb300")
+
+FAKE = 1 << 40
+ES = {"f32": 4, "f64": 8, "c64": 8, "c128": 16}
+
+
+def _layout(spec, dtype, shift=0):
+    ptrs = FAKE + spec.buf.astype(np.int64) * (1 << 32) + (spec.off + shift) * ES[dtype]
+    return costa.costa_layout_from_spec(spec, dtype, ptrs)
+
+
+def _tile_moves(tiles, es):
+    out = []
+    for t in tiles:
+        x, y = np.meshgrid(np.arange(t["nx"], dtype=np.int64), np.arange(t["ny"], dtype=np.int64))
+        d = int(t["dst"]) + (x + y * int(t["dld"])) * es
+        s = int(t["src"]) + ((x * int(t["sld"]) + y) if t["flags"] & 1 else (x + y * int(t["sld"]))) * es
+        out.append(np.stack([d.ravel(), s.ravel()]))
+    return np.concatenate(out, axis=1) if out else np.zeros((2, 0), np.int64)
+
+
+def _patch_moves(patches, cells, es):
+    ext = 16 if es == 16 else 32
+    out = []
+    for p in patches:
+        nx, ny, lm, rm = int(p["nx"]), int(p["ny"]), int(p["lmask"]), int(p["rmask"])
+        assert 1 <= nx <= ext and 1 <= ny <= ext
+        tr = bool(p["flags"] & 1)
+        nl, nr = (ny, nx) if tr else (nx, ny)
+        assert lm & 1 and rm & 1 and lm < 1 << nl and rm < 1 << nr
+        nls, nrs = bin(lm).count("1"), bin(rm).count("1")
+        assert nls <= 8 and nrs <= 8
+        seg = lambda m, i: bin(m & ((2 << i) - 1)).count("1") - 1
+        ls = np.array([seg(lm, i) for i in range(nl)])
+        rs = np.array([seg(rm, i) for i in range(nr)])
+        c = cells[int(p["cell0"]):int(p["cell0"]) + nls * nrs]
+        assert len(c) == nls * nrs
+        r, l = np.meshgrid(np.arange(nr), np.arange(nl), indexing="ij")
+        k = rs[r] * nls + ls[l]
+        # biased addresses wrap modulo 2^64
+        s = (c["src"][k] + ((r * c["sld"].astype(np.int64)[k] + l) * es).astype(np.uint64)).astype(np.int64)
+        x, y = (r, l) if tr else (l, r)
+        d = int(p["dst"]) + (x + y * int(p["dld"])) * es
+        out.append(np.stack([d.ravel(), s.ravel()]))
+    return np.concatenate(out, axis=1) if out else np.zeros((2, 0), np.int64)
+
+
+def _same(a, b):
+    a, b = (m[:, np.lexsort((m[1], m[0]))] for m in (a, b))
+    return np.array_equal(a, b)
+
+
+def check(p, shift=0):
+    """True when the pair has patches (and they were checked)."""
+    LA, LB = _layout(p.A, p.dtype, shift), _layout(p.B, p.dtype, shift)
+    try:
+        patches, cells = costa.costa_debug_patches(LA, LB, p.op)
+        tiles = costa.costa_debug_tiles(LA, LB, p.op)
+    finally:
+        LA.destroy()
+        LB.destroy()
+    one = lambda s: len(set(s.order[i, j] for i in range(s.nbr) for j in range(s.nbc)
+                            if s.rsplit[i + 1] > s.rsplit[i] and s.csplit[j + 1] > s.csplit[j])) <= 1
+    if not one(p.A) or not one(p.B):
+        assert len(patches) == 0
+        return False
+    es = ES[p.dtype]
+    got = _patch_moves(patches, cells, es)
+    assert got.shape[1] == p.A.m * p.A.n
+    assert _same(got, _tile_moves(tiles, es))
+    conj = p.op == "C"
+    assert np.all(((patches["flags"] & 4) != 0) == conj)
+    return len(patches) > 0
+
+
+def test_fuzz_and_small_blocks():
+    seen = sum(check(C.fuzz_problem(k, max_dim=90)) for k in range(160))
+    assert seen > 10  # both sides block-cyclic (one element order each): about one in nine
+    assert all(check(C.small_block_problem(k)) for k in range(96))
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f64", "c128"])
+@pytest.mark.parametrize("op", ["N", "T", "C"])
+@pytest.mark.parametrize("storage", ["CC", "CR", "RC", "RR"])
+def test_block_cyclic_forms(dtype, op, storage):
+    """Grids from 1 x 1 (where the blocks of both sides join) to 2 x 3, block
+    sizes that divide each other and that do not, odd leading dimensions and
+    base addresses, both storage orders."""
+    m, n = 83, 101
+    for (mb, nb), (ma, na), (pr, pc), pad, shift in (((5, 7), (3, 4), (1, 1), 0, 0), ((50, 50), (75, 75), (2, 2), 1, 1),
+                                                     ((1, 1), (2, 3), (2, 3), 3, 0), ((8, 8), (4, 16), (3, 2), 0, 1),
+                                                     ((33, 65), (32, 32), (2, 1), 2, 0)):
+        bm, bn = (m, n) if op == "N" else (n, m)
+        B = L.block_cyclic(bm, bn, mb, nb, pr, pc, storage=storage[1], ld_pad=pad, name="B")
+        A = L.block_cyclic(m, n, ma, na, pr, pc, grid_order="C", storage=storage[0], ld_pad=1 - pad % 2, name="A")
+        assert check(C.Problem("patch", dtype, op, 1.0, 0.0, A, B), shift)
+
+
+def test_joined_blocks_make_few_cells():
+    """On 1 x 1 grids every block continues its neighbours in storage, so a
+    whole patch is one cell whatever the block sizes."""
+    B = L.block_cyclic(128, 96, 5, 7, 1, 1, name="B")
+    A = L.block_cyclic(96, 128, 3, 4, 1, 1, name="A")
+    LA, LB = _layout(A, "f64"), _layout(B, "f64")
+    patches, cells = costa.costa_debug_patches(LA, LB, "T")
+    assert len(patches) == 3 * 4 and len(cells) == len(patches)
+    assert np.all(patches["nx"] == 32) and np.all(patches["ny"] == 32)
