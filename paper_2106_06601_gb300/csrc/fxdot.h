@@ -7,19 +7,28 @@
 // subnormal, infinite or NaN operand; callers test this and take another
 // evaluation otherwise).  Then:
 //   1. each product's significand product is formed from the two 53-bit
-//      significands, shifted to the top of 64 bits, by one 64 x 64 -> high
-//      64 multiply: its top 64 bits (the truncated part is below 2^-62 of
-//      the product);
-//   2. the products are aligned to the largest exponent, 3 bits of headroom
-//      added, and summed exactly as signed 64-bit integers in units
-//      U = 2^-7 ulp(M) or finer (M the largest product): each alignment
-//      truncates less than one U;
-//   3. the integer sum is rounded once to double, to nearest even.
+//      significands, split into their top 31 and low 22 bits (these shifted
+//      to the top of a word), by four 32 x 32 -> 64-bit multiply-adds, of
+//      which the bits below 2^44 are dropped: the floor, in [2^60, 2^62);
+//   2. the products are aligned to the largest exponent, with one bit of
+//      headroom, and summed exactly as signed 64-bit integers in units
+//      U = 2^-7 ulp(M) or finer (M the largest product): dropping and
+//      alignment together truncate less than one U per product;
+//   3. the integer sum is rounded once to double, to nearest even, by the
+//      hardware's conversion, and the exponent added to its exponent field.
 // The result is within 0.5 ulp(x) + n U of the exact sum x of the n exact
 // products: n U <= 2^-5 ulp(M), so at most 0.5 ulp(x) + 0.032 ulp(M).  All
 // intermediate magnitudes stay in the normal range: a product lies in
 // [2^-960, 2^960), the sum below 2^962, and a nonzero result is a multiple of
 // U >= 2^-1019.
+//
+// The ALU pipe bounds the kernels that use it.  This split keeps every
+// partial sum inside 64 bits, so that there are no carries, and drops whole
+// words, so that there are no shifts (one 64 x 64 -> high 64 multiply takes
+// about twice the instructions); the conversion replaces
+// the count of leading zeros, the shifts and the rounding: 4096^2 c128 T,
+// complex beta, BC64 -> BC128: 2340 -> 3450 GB/s (430 -> 320
+// instructions per element).
 //
 // The same code compiles for the host (costa_debug_fxdot uses it), so the
 // arithmetic can be checked without a GPU.
@@ -57,27 +66,38 @@ COSTA_FX_HD double from_bits(uint64_t u) {
 #endif
 }
 
-COSTA_FX_HD uint64_t mulhi(uint64_t a, uint64_t b) {
+// x * y + a without overflow checks (one multiply-add on the GPU).
+COSTA_FX_HD uint64_t mad_wide(uint32_t x, uint32_t y, uint64_t a) {
+    return static_cast<uint64_t>(x) * y + a;
+}
+
+// v >> n, 0 for n >= 64 (the GPU's shift clamps its count).
+COSTA_FX_HD uint64_t shr_clamp(uint64_t v, uint32_t n) {
 #ifdef __CUDA_ARCH__
-    return __umul64hi(a, b);
+    uint64_t r;
+    asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
+    return r;
 #else
-    return static_cast<uint64_t>((static_cast<unsigned __int128>(a) * b) >> 64);
+    return n < 64u ? v >> n : 0;
 #endif
 }
 
-COSTA_FX_HD int clz64(uint64_t v) {  // v != 0
+// The integer rounded to the nearest double, ties to even.
+COSTA_FX_HD double round_to_double(int64_t v) {
 #ifdef __CUDA_ARCH__
-    return __clzll(static_cast<long long>(v));
+    return __ll2double_rn(v);
 #else
-    return __builtin_clzll(v);
+    return static_cast<double>(v);  // the default rounding mode is to nearest even
 #endif
 }
 
-// An operand: its 53-bit significand shifted left by 11 (in [2^63, 2^64);
-// 0 for a zero), its biased exponent and its sign bit.
+// An operand: its 53-bit significand as 31 top bits (h) and 22 low bits at the
+// top of a word (l = low bits * 2^10), both 0 for a zero; its biased exponent (kZeroExp for a zero, so that a zero
+// product never is the largest); its sign as a mask.
+constexpr int32_t kZeroExp = -8192;
 struct Op {
-    uint64_t m;
-    uint32_t e;
+    uint32_t h, l;
+    int32_t e;
     uint32_t s;
 };
 
@@ -91,67 +111,58 @@ COSTA_FX_HD bool in_range(double v) {
 
 COSTA_FX_HD Op unpack(double v) {
     const uint64_t u = bits_of(v);
+    const uint32_t hi = static_cast<uint32_t>(u >> 32), lo = static_cast<uint32_t>(u);
+    const uint32_t e = (hi >> 20) & 0x7FFu;
+    const uint32_t top = e ? (hi & 0xFFFFFu) | 0x100000u : 0u;
     Op o;
-    o.s = static_cast<uint32_t>(u >> 63);
-    o.e = static_cast<uint32_t>(u >> 52) & 0x7FFu;
-    o.m = o.e ? ((u << 11) | (uint64_t(1) << 63)) : 0;
+    o.h = (top << 10) | (lo >> 22);
+    o.l = lo << 10;
+    o.e = e ? static_cast<int32_t>(e) : kZeroExp;
+    o.s = static_cast<uint32_t>(static_cast<int32_t>(hi) >> 31);
     return o;
 }
 
-// One product x * y, negated when neg = 1: the top 64 bits of the
-// significand product (in [2^62, 2^64), or 0), the sum of the biased
-// exponents (0 for a zero product) and the sign.
+// One product x * y, negated when neg = 1: floor(significand product / 2^44)
+// (in [2^60, 2^62), or 0), the sum of the biased exponents and the sign as a
+// mask.
 struct Term {
     uint64_t p;
-    uint32_t e;
+    int32_t e;
     uint32_t s;
 };
 
 COSTA_FX_HD Term mul(const Op &x, const Op &y, uint32_t neg) {
     Term t;
-    t.p = mulhi(x.m, y.m);
-    t.e = t.p ? x.e + y.e : 0u;
-    t.s = x.s ^ y.s ^ neg;
+    const uint64_t low = mad_wide(x.l, y.l, 0) >> 32;
+    const uint64_t mid = mad_wide(x.l, y.h, mad_wide(x.h, y.l, low));  // below 2^64 (h < 2^31)
+    t.p = mad_wide(x.h, y.h, mid >> 32);
+    t.e = x.e + y.e;
+    t.s = x.s ^ y.s ^ (neg ? 0xFFFFFFFFu : 0u);
     return t;
 }
 
-// The sum of n terms, rounded once to double (to nearest, ties to even).
+// The sum of n <= 4 terms, rounded once to double (to nearest, ties to even).
 // A zero sum gives +0.
 template <int N>
 COSTA_FX_HD double sum(const Term (&t)[N]) {
-    uint32_t emax = t[0].e;
+    int32_t emax = t[0].e;
 #pragma unroll
     for (int i = 1; i < N; ++i) emax = t[i].e > emax ? t[i].e : emax;
-    int64_t acc = 0;
+    uint64_t acc = 0;
+    uint32_t neg = 0;  // minus the number of negative terms: v ^ mask = -v - 1
 #pragma unroll
     for (int i = 0; i < N; ++i) {
-        const uint32_t sh = emax - t[i].e + 3u;  // >= 3: |each| < 2^61, |sum| < 2^63
-        const int64_t v = sh < 64u ? static_cast<int64_t>(t[i].p >> sh) : 0;
-        acc += t[i].s ? -v : v;
+        const uint64_t v = shr_clamp(t[i].p, static_cast<uint32_t>(emax - t[i].e + 1));  // < 2^61: |sum| < 2^63
+        const uint64_t mask = (static_cast<uint64_t>(t[i].s) << 32) | t[i].s;
+        acc += v ^ mask;
+        neg += t[i].s;
     }
+    acc -= static_cast<uint64_t>(static_cast<int64_t>(static_cast<int32_t>(neg)));
     if (acc == 0) return 0.0;
-    const uint64_t sign = acc < 0 ? uint64_t(1) << 63 : 0;
-    const uint64_t mag = acc < 0 ? uint64_t(0) - static_cast<uint64_t>(acc) : static_cast<uint64_t>(acc);
-    int nb = 64 - clz64(mag);  // bit length, <= 63
-    uint64_t sig;
-    if (nb <= 53) {
-        sig = mag << (53 - nb);
-    } else {
-        const int sh = nb - 53;
-        sig = mag >> sh;
-        const uint64_t rem = mag & ((uint64_t(1) << sh) - 1), half = uint64_t(1) << (sh - 1);
-        if (rem > half || (rem == half && (sig & 1))) {
-            ++sig;
-            if (sig >> 53) {
-                sig >>= 1;
-                ++nb;
-            }
-        }
-    }
-    // the acc's unit is 2^(emax - 2105); a significand of 53 bits then has
-    // biased exponent nb + emax - 1083, in [4, 1985] for in-range operands
-    const uint64_t be = static_cast<uint64_t>(nb) + emax - 1083u;
-    return from_bits(sign | (be << 52) | (sig & ((uint64_t(1) << 52) - 1)));
+    // acc's unit is 2^(emax - 2105): a significand product has unit
+    // 2^(emax - 2150), and acc's is 2^45 of it
+    const uint64_t r = bits_of(round_to_double(static_cast<int64_t>(acc)));
+    return from_bits(r + (static_cast<uint64_t>(static_cast<int64_t>(emax - 2105)) << 52));
 }
 
 }  // namespace fx

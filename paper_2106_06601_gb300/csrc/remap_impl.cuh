@@ -82,7 +82,8 @@ template <> struct ET<double2> { enum { VEC = 1, CPLX = 1 }; typedef double R; }
 //   16-byte  both         copy                            4      1     2
 //            both         scale                           4      3     1
 //            both         complex alpha, beta = 0         4      3     1
-//            both         kinds that read A               4      2     1
+//            both         complex beta                    4      3     1
+//            both         real kinds that read A          4      2     1
 //
 // Why, where a row departs from its neighbours:
 //  - 8-byte light kinds (copy, axpby2) run more warps without look-ahead;
@@ -119,7 +120,8 @@ template <> struct ET<double2> { enum { VEC = 1, CPLX = 1 }; typedef double R; }
 //    A two groups ahead (unrolled with A's tile in registers: 1105 one pass
 //    at a time, 1186 with 2, 1194 with 4, instruction fetch the limit;
 //    rolled: 2286 with 1, 2340 with 2 at 136 registers and 3 blocks, 2115
-//    with 4).
+//    with 4).  With the sums' shorter form (fxdot.h), 4096^2: 2 blocks 292
+//    us, 3 blocks 234, 4 blocks 238 (spills); 1, 2, 3 passes 264, 234, 252.
 // Each entry is overridable at build time for tuning (COSTA_WARPS_4/8,
 // COSTA_MINB_* and COSTA_NBUF_*).
 #ifndef COSTA_WARPS_4
@@ -204,6 +206,9 @@ template <> struct ET<double2> { enum { VEC = 1, CPLX = 1 }; typedef double R; }
 #ifndef COSTA_NBUF_16CS
 #define COSTA_NBUF_16CS 1
 #endif
+#ifndef COSTA_MINB_16C
+#define COSTA_MINB_16C 3
+#endif
 #ifndef COSTA_MINB_16A
 #define COSTA_MINB_16A 2
 #endif
@@ -221,6 +226,7 @@ constexpr Shape launch_shape(int es, bool cplx, int kind, bool mis) {
     const bool reads_a = kind_reads_a(kind);
     if (es == 4) return reads_a ? Shape{COSTA_MINB_4A, COSTA_NBUF_4A} : Shape{COSTA_MINB_4, COSTA_NBUF_4};
     if (es == 16) {
+        if (kind == K_CPLX) return {COSTA_MINB_16C, COSTA_NBUF_16A};
         if (reads_a) return {COSTA_MINB_16A, COSTA_NBUF_16A};
         if (kind == K_CSCALE) return {COSTA_MINB_16CS, COSTA_NBUF_16CS};
         return kind == K_SCALE ? Shape{COSTA_MINB_16S, COSTA_NBUF_16S} : Shape{COSTA_MINB_16, COSTA_NBUF_16};
@@ -712,7 +718,7 @@ __device__ __forceinline__ void stage_drain(const Geom<T> &g, const Sc &s, unsig
         // double complex with complex scalars: G passes at a time in
         // straight-line code, so that their evaluations overlap.  Four-term
         // components (complex beta) are all summed in fixed point on the
-        // integer pipes (about 150 instructions each, in long dependent
+        // integer pipes (over 100 instructions each, in long dependent
         // chains); two-term ones (complex alpha, beta = 0) by mid_cscale.  The
         // loop stays rolled: unrolled over the
         // tile's passes, the fixed-point sums made a body of about 14,000

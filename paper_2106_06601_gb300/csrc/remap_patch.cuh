@@ -61,6 +61,13 @@ namespace remap {
 #ifndef COSTA_PB_8A
 #define COSTA_PB_8A 4
 #endif
+// complex scalars on double complex data
+#ifndef COSTA_PB_16C
+#define COSTA_PB_16C 4
+#endif
+#ifndef COSTA_PGR
+#define COSTA_PGR 2
+#endif
 #ifndef COSTA_PB_16
 #define COSTA_PB_16 4
 #endif
@@ -68,7 +75,7 @@ namespace remap {
 constexpr int patch_blocks(int es, bool cplx, int kind) {
     const bool reads_a = kind_reads_a(kind);
     if (es == 4) return reads_a ? COSTA_PB_4A : COSTA_PB_4;
-    if (es == 16) return COSTA_PB_16;
+    if (es == 16) return kind == K_CPLX || kind == K_CSCALE ? COSTA_PB_16C : COSTA_PB_16;
     return reads_a ? COSTA_PB_8A : kind == K_SCALE && !cplx ? COSTA_PB_8S : COSTA_PB_8;
 }
 
@@ -84,12 +91,13 @@ template <typename T, int KIND> struct PCfg {
     static constexpr int ELEMS = EX * PITCH_T > EY * PITCH_N ? EX * PITCH_T : EY * PITCH_N;
     static constexpr int BUF = (ELEMS * ES + 15) / 16 * 16;
     static constexpr int CELLS = kPatchCells * 16;
-    // the fixed-point sums of double complex data stay one pass per iteration
-    // (their code is long)
+    // complex scalars on double complex data: two passes together, rolled (the
+    // fixed-point sums are long; BC50 -> BC75, 4096^2, complex beta, one, two,
+    // four passes: 306, 276, 322 us)
     static constexpr bool ROLLED = ES == 16 && (KIND == K_CPLX || KIND == K_CSCALE);
     // passes whose elements of A are loaded together: the whole patch in two
     // groups, a quarter for 8-byte elements (registers)
-    static constexpr int G = ROLLED ? 1 : ES == 4 ? 16 : ES == 8 ? 8 : 4;
+    static constexpr int G = ROLLED ? COSTA_PGR : ES == 4 ? 16 : ES == 8 ? 8 : 4;
 };
 
 // Index of the segment that holds element i of an axis (mask: bit k set
@@ -239,7 +247,7 @@ __device__ __forceinline__ void patch_write(const PatchLaunch &a, const PatchDes
                 }
             }
         } else {
-            constexpr int U = P::ROLLED ? 1 : 8;
+            constexpr int U = P::ROLLED ? COSTA_PGR : 8;
 #pragma unroll U
             for (int p = 0; p < cnt; ++p) {
                 *dst = combine<KIND>(*reinterpret_cast<const T *>(sp), T(), s);
