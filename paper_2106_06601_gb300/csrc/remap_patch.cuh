@@ -27,6 +27,7 @@
 #pragma once
 
 #include "remap_impl.cuh"
+#include "rnmul.h"
 
 namespace costa {
 namespace remap {
@@ -87,6 +88,9 @@ template <typename T, int KIND> struct PCfg {
     static constexpr int PITCH_T = EY + 1, PITCH_N = EX + 1;
     static constexpr int WARPS = COSTA_PW;
     static constexpr bool READS_A = kind_reads_a(KIND);
+    // real doubles: part of the products beta * a and alpha * b are formed on
+    // the integer pipes (mul_group)
+    static constexpr bool INT_MUL = sizeof(T) == 8 && !ET<T>::CPLX;
     static constexpr int MINB = patch_blocks(ES, ET<T>::CPLX != 0, KIND);
     static constexpr int ELEMS = EX * PITCH_T > EY * PITCH_N ? EX * PITCH_T : EY * PITCH_N;
     static constexpr int BUF = (ELEMS * ES + 15) / 16 * 16;
@@ -187,6 +191,33 @@ __device__ __forceinline__ void patch_stage(const PatchDesc &d, const uint4 *cel
     }
 }
 
+// Multiplies the doubles of a group by c, each product rounded to nearest:
+// every other one on the integer pipes (rnmul.h), the others on the FP64
+// pipe; all of them there when some lane of the warp holds a value that the
+// integer form does not admit (one vote, so that no predicated-off FP64
+// instruction is issued).  GB300, 8192^2, none / every fourth / every other /
+// all of them on the integer pipes, us per call: f64 T beta = 0.7 BC50 -> BC75
+// 293 / 294 / 287 / 294, odd lds 295 / 295 / 287 / 288, T alpha = 1.5 BC50 ->
+// BC75 206 / 187 / 192 / 240.  c128 (half the values per row) loses 5%.
+template <typename T, int N>
+__device__ __forceinline__ void mul_group(Chunk<T> (&v)[N], double c, unsigned mask) {
+    double *d = reinterpret_cast<double *>(v);
+    const rn::Factor f = rn::factor(c);
+    bool bad = false;
+#pragma unroll
+    for (int k = 1; k < 2 * N; k += 2) bad |= !rn::admits(f, d[k]);
+    const bool all_fp64 = __any_sync(mask, bad);
+#pragma unroll
+    for (int k = 0; k < 2 * N; k += 2) d[k] = __dmul_rn(c, d[k]);
+    if (all_fp64) {
+#pragma unroll
+        for (int k = 1; k < 2 * N; k += 2) d[k] = __dmul_rn(c, d[k]);
+    } else {
+#pragma unroll
+        for (int k = 1; k < 2 * N; k += 2) d[k] = rn::mul(f, d[k]);
+    }
+}
+
 // Writes a staged patch to A in A's contiguous order, one element per lane.
 template <typename T, int KIND>
 __device__ __forceinline__ void patch_write(const PatchLaunch &a, const PatchDesc &d, Sc &s, int &cached,
@@ -222,9 +253,10 @@ __device__ __forceinline__ void patch_write(const PatchLaunch &a, const PatchDes
     };
     auto write = [&](Chunk<T> (&v)[NC], int p0) {
         if (KIND == K_AXPBY2) prescale<T>(v, NC, s, mask);
+        if constexpr (KIND == K_AXPBY && P::INT_MUL) mul_group<T>(v, s.br, mask);  // beta * a, then as K_AXPBY2
 #pragma unroll
         for (int k = 0; k < G; ++k) {
-            if (p0 + k < cnt) *dst = combine<KIND>(*reinterpret_cast<const T *>(sp), v[k / V].e[k % V], s);
+            if (p0 + k < cnt) *dst = combine<KIND == K_AXPBY && P::INT_MUL ? K_AXPBY2 : KIND>(*reinterpret_cast<const T *>(sp), v[k / V].e[k % V], s);
             dst += step;
             sp += sstep;
         }
@@ -244,6 +276,24 @@ __device__ __forceinline__ void patch_write(const PatchLaunch &a, const PatchDes
                 if (p0 + G < npass) {
                     write(av[1], p0 + G);
                     if (p0 + 3 * G < npass) load(av[1], p0 + 3 * G);
+                }
+            }
+        } else if constexpr (KIND == K_SCALE && P::INT_MUL) {
+#pragma unroll 1
+            for (int p0 = 0; p0 < npass; p0 += G) {  // uniform across the lanes in `mask`
+                Chunk<T> (&v)[NC] = av[0];
+#pragma unroll
+                for (int k = 0; k < G; ++k) {
+                    T e = T();
+                    if (p0 + k < cnt) e = *reinterpret_cast<const T *>(sp);
+                    v[k / V].e[k % V] = e;
+                    sp += sstep;
+                }
+                mul_group<T>(v, s.ar, mask);
+#pragma unroll
+                for (int k = 0; k < G; ++k) {
+                    if (p0 + k < cnt) *dst = combine<K_COPY>(v[k / V].e[k % V], T(), s);
+                    dst += step;
                 }
             }
         } else {

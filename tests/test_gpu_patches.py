@@ -42,6 +42,53 @@ def test_edges_of_patches(dtype, op, dev):
             check_problem(p, dev, guard=2)
 
 
+def _special_doubles(n, rng):
+    """Random doubles with all exponents, exact halfway products, zeros,
+    subnormals, infinities and NaNs among runs of ordinary values."""
+    import numpy as np
+
+    v = rng.standard_normal(n)
+    k = n // 4  # ordinary runs stay: whole warps without a special value
+    at = k + rng.permutation(n - k)[:k]
+    bits = rng.integers(0, 1 << 63, k, dtype=np.uint64) | (rng.integers(0, 2, k, dtype=np.uint64) << np.uint64(63))
+    v[at] = bits.view(np.float64)
+    few = at[:k // 2]
+    v[few] = np.ldexp(np.round(np.ldexp(rng.random(len(few)), 20)), rng.integers(-1070, 1000, len(few)))  # few bits: exact
+    v[at[:64]] = np.resize([0.0, -0.0, np.inf, -np.inf, np.nan, 5e-324, -2.2e-308, 1.7e308], 64)
+    return v
+
+
+@pytest.mark.parametrize("factor", [0.7, -3.0, 1.0 + 2.0 ** -52, 1.5e-300, 7e250, 5e-324])
+@pytest.mark.parametrize("scale", [True, False])
+def test_products_of_doubles_are_rounded_once(factor, scale, dev):
+    """beta * a (with a zero B) and alpha * b equal numpy's products bit for
+    bit, whichever pipe forms them."""
+    import numpy as np
+
+    from tests._gpu import OnDevice, block_mask
+    from tests._util import global_matrix
+    from workloads.materialize import HostMatrix
+
+    B = L.block_cyclic(300, 210, 50, 50, 2, 2, name="B")
+    A = L.block_cyclic(210, 300, 75, 75, 2, 2, name="A")
+    alpha, beta = (factor, 0.0) if scale else (1.0, factor)
+    p = C.Problem("rn", "f64", "T", alpha, beta, A, B)
+    rng = np.random.default_rng(7)
+    hb, ha = HostMatrix(B, "f64"), HostMatrix(A, "f64")
+    (hb if scale else ha).arena[...] = _special_doubles((hb if scale else ha).arena.size, rng)
+    g = OnDevice(p, dev, B_host=hb, A_host=ha)
+    g.run()
+    got = g.Ad.download()
+    g.close()
+    with np.errstate(all="ignore"):
+        want = factor * global_matrix(B, hb.buffers()).real.T if scale else factor * global_matrix(A, ha.buffers()).real + 0.0
+    G = global_matrix(A, got.buffers()).real
+    same = (G.view(np.int64) == np.ascontiguousarray(want).view(np.int64)) | (np.isnan(G) & np.isnan(want))
+    assert np.all(same), np.argwhere(~same)[:3]
+    mask = block_mask(A, ha)
+    assert np.array_equal(got.arena[~mask], ha.arena[~mask], equal_nan=True)
+
+
 def test_batch_of_tiles_and_patches(dev):
     """One batch whose problems differ in kind, op and work list: layouts with
     mixed element orders stay with the tile kernels."""
