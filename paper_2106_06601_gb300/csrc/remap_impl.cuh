@@ -83,7 +83,7 @@ template <> struct ET<double2> { enum { VEC = 1, CPLX = 1 }; typedef double R; }
 //            both         scale                           4      3     1
 //            both         complex alpha, beta = 0         4      3     1
 //            both         complex beta                    4      3     1
-//            both         real kinds that read A          4      2     1
+//            both         real kinds that read A          4      3     1
 //
 // Why, where a row departs from its neighbours:
 //  - 8-byte light kinds (copy, axpby2) run more warps without look-ahead;
@@ -113,8 +113,8 @@ template <> struct ET<double2> { enum { VEC = 1, CPLX = 1 }; typedef double R; }
 //    warps per SM leave exposed; 4 buffers lost 20-40%.
 //  - 8-byte element path (misaligned, kinds that read A): a whole tile of A
 //    in registers, which 4 blocks fit without spills.
-//  - 16-byte kinds that read A hold a whole 16 KB tile of A in registers,
-//    except with a complex beta: there each component is a fixed-point sum
+//  - 16-byte kinds that read A pass it through registers in groups
+//    (write_grouped), except with a complex beta: there each component is a fixed-point sum
 //    on the integer pipes (498 GB/s with Dot2 on the FP64 pipe), and the
 //    drain is a rolled loop over COSTA_FX_GROUP passes at a time that loads
 //    A two groups ahead (unrolled with A's tile in registers: 1105 one pass
@@ -210,7 +210,7 @@ template <> struct ET<double2> { enum { VEC = 1, CPLX = 1 }; typedef double R; }
 #define COSTA_MINB_16C 3
 #endif
 #ifndef COSTA_MINB_16A
-#define COSTA_MINB_16A 2
+#define COSTA_MINB_16A 3
 #endif
 #ifndef COSTA_NBUF_16A
 #define COSTA_NBUF_16A 1
@@ -1421,6 +1421,67 @@ __device__ __forceinline__ void stage_any(const Geom<T> &g, unsigned char *buf, 
     else if (g.fast) stage_issue<T>(g, buf, lane);  // the element-wise fallback stages nothing
 }
 
+// 16-byte elements and real scalars with beta != 0: an aligned tile whose A
+// chunks pass through registers in groups of G passes, two groups ahead of the
+// one that is combined (the first two are loaded before the wait for the
+// source).  A whole 16 KB tile of A takes 128 registers per lane and leaves
+// two blocks per SM; the groups leave three, the most that shared memory fits.
+// GB300, 6016^2, BC64 -> BC128, us per call, whole tile / groups of 2, 4, 8
+// passes: N beta = 0.5 287 / 409, 300, 271; T beta = 0.7 332 / 384, 332, 323.
+template <typename T, int KIND> __host__ __device__ constexpr bool grouped_a() {
+    return sizeof(T) == 16 && (KIND == K_AXPBY || KIND == K_AXPBY2);
+}
+template <typename T, int KIND, int NB>
+__device__ __forceinline__ void write_grouped(const Geom<T> &g, const Sc &s, unsigned char *buf, int lane) {
+    constexpr int G = 8;
+    const LaneMap m = lane_map(g.nx, lane);
+    const bool on = m.c < g.nx;
+    const unsigned mask = __ballot_sync(0xffffffffu, on);
+    const int cnt = g.ny > m.r0 ? (g.ny - m.r0 + m.rpp - 1) / m.rpp : 0;  // passes of this lane
+    const int npass = (g.ny + m.rpp - 1) / m.rpp;
+    T *dst = g.dst + m.c + static_cast<int64_t>(m.r0) * g.dld;
+    const T *q = dst;
+    const int64_t step = static_cast<int64_t>(m.rpp) * g.dld;
+    Chunk<T> av[2][G];
+    auto load = [&](Chunk<T> (&v)[G], int p0) {
+#pragma unroll
+        for (int k = 0; k < G; ++k) {
+            v[k].raw = make_uint4(0, 0, 0, 0);
+            if (p0 + k < cnt) v[k] = load_rw(q);
+            q += step;
+        }
+    };
+    auto write = [&](Chunk<T> (&v)[G], int p0) {
+        if (KIND == K_AXPBY2) prescale<T>(v, G, s, mask);
+#pragma unroll
+        for (int k = 0; k < G; ++k) {
+            if (p0 + k < cnt) {
+                const int y = (p0 + k) * m.rpp + m.r0;
+                const T b = *reinterpret_cast<const T *>(g.transpose ? slot<T>(buf, m.c, y) : slot<T>(buf, y, m.c));
+                *dst = combine<KIND>(b, v[k].e[0], s);
+            }
+            dst += step;
+        }
+    };
+    if (on) {
+        load(av[0], 0);
+        load(av[1], G);
+    }
+    cp_async_wait<NB - 1>();
+    __syncwarp();
+    if (on) {
+#pragma unroll 1
+        for (int p0 = 0; p0 < npass; p0 += 2 * G) {
+            write(av[0], p0);
+            if (p0 + 2 * G < npass) load(av[0], p0 + 2 * G);
+            if (p0 + G < npass) {
+                write(av[1], p0 + G);
+                if (p0 + 3 * G < npass) load(av[1], p0 + 3 * G);
+            }
+        }
+    }
+}
+
 // Writes one staged tile.  `cached` holds the problem whose scalars are in
 // `s`.
 template <typename T, int KIND, int NB, bool MIS>
@@ -1443,6 +1504,8 @@ __device__ __forceinline__ void write_tile(const RemapLaunch &a, const Geom<T> &
         __syncwarp();
         if (sizeof(T) == 4 && g.elem) stage_drain_e1<T, KIND>(g, s, buf, lane);
         else stage_drain_w<T, KIND>(g, s, buf, lane);
+    } else if (grouped_a<T, KIND>() && g.fast) {
+        if constexpr (grouped_a<T, KIND>()) write_grouped<T, KIND, NB>(g, s, buf, lane);
     } else if (g.fast) {
         Chunk<T> av[C::NPASS];
         if constexpr (!drain_loads_a<T, KIND>()) load_a<T, KIND>(g, s, av, lane);
