@@ -362,18 +362,29 @@ costa_status check_access(costa_layout_s *L, int dev, const char *which) {
     return check_access_impl(L, dev, which, nullptr, 0);
 }
 
-// Moves the problems that the patch kernel serves from the tile list to
-// patches: every problem that has patches, when at least half of the list's
-// elements lie in small or misaligned tiles (4-byte tiles whose target runs
-// are aligned count as aligned: their window path is the faster one).
+// The patches of a plan, for two reasons.
+//
+// 1. At least half of the list's elements lie in tiles that are small,
+// misaligned (4-byte tiles whose target runs are aligned count as aligned:
+// their window path is the faster one) or, for 8- and 16-byte elements, less
+// than three quarters of a full tile; or, for 8-byte elements, a twentieth lie
+// in misaligned tiles (two launches, and the halves of the lines where they
+// meet apart): every problem that has patches moves from the tile list to
+// patches, for every kind.
 // Measured on GB300, same box, 8192^2 (c128 6016^2), us per call, tile and
 // small-tile kernels -> patch kernel:
 //   BC50 -> BC75   f64 T copy 226 -> 175, N copy 231 -> 172, T beta = 0.5
 //                  312 -> 265, T beta = 0.7 494 -> 293; f32 T copy 212 ->
-//                  108; c64 T beta = 0.7 464 -> 261; c128 T copy 224 -> 190
+//                  108; c64 T beta = 0.7 464 -> 261; c128 T copy 224 -> 190,
+//                  beta = 0.5 341 -> 280
+//   partial tiles  c128 BC37 -> BC128 N copy 297 -> 188, BC24 -> BC100 T copy
+//                  266 -> 184; f64 BC24 -> BC100 T copy 220 -> 214 (f32 109 ->
+//                  116, which stays)
 //   odd lds, T     f64 copy 210 -> 191, beta = 0.7 408 -> 293 (A's ld odd:
 //                  copy 182 -> 166, beta = 0.5 250 -> 250); f32, A's ld odd,
 //                  copy 112 -> 109, beta = 0.5 157 -> 149
+//   a quarter misaligned (7001 x 6003, BC64): f64 T copy 116 -> 104, N beta =
+//                  0.5 177 -> 161
 //   BC4 (half the rows), T copy: f64 290 -> 83, f32 310 -> 53, c64 299 ->
 //                  83, c128 191 -> 92
 //   BC8, T         f64 copy 187 -> 162, beta = 0.5 258 -> 242; f32 copy 164
@@ -382,33 +393,83 @@ costa_status check_access(costa_layout_s *L, int dev, const char *which) {
 //   BC16, T        f64 copy 182 -> 161; f32 copy 112 -> 101, beta = 0.5 146
 //                  -> 139; c128 beta = 0.5 375 -> 266
 // f32 with only B's ld odd: copy 99 -> 105 (kept on the window path).
+//
+// 2. Aligned lists of 8-byte elements with more data than the L2 cache holds
+// and targets that are not one contiguous run per tile: the kinds in
+// kAlignedPatchKinds run on patches (if every problem has them), the other
+// f64 kinds on the tiles, unless some are misaligned (two or three launches: a
+// submatrix, 6001 x 4999, 2% misaligned, T beta = 0.7 150 -> 134) or, for the
+// general beta, TMA could stage less than three quarters of them.  Same box, 8192^2, BC64 -> BC128, tiles -> patches:
+// f64 T copy 172 -> 162, T beta = 0.5 250 -> 242, N beta = 0.5 257 -> 242, but
+// alpha = 1.5 171 -> 176 and beta = 0.7 263 (TMA) -> 271; c64 T copy 171 ->
+// 161, N beta = 0.5 265 -> 241, T beta = 0.7 246 -> 242, complex beta 293 ->
+// 277.  4096^2 f64 T copy 46.3 -> 44.5; 2048^2 (in L2) 13.4 -> 14.6.  Targets
+// of 16-row panels (one run per tile) 1900 -> 1885 with three times the list.
+// c128: copy 1321 -> 1329 (16384^2), f32: copy 88 -> 103, stay on the tiles.
 // COSTA_PATCH=0 turns the patches off, COSTA_PATCH=1 takes them for every
 // pair that has them (for measurements).
-void take_patches(const Plan &plan, std::vector<TileDesc> &list, PatchList &out) {
+// Returns the kinds that run on patches (bit per kind; 0: no patches).
+// `rest`: the tiles left in `list` are other problems' than the patches'
+// (reason 1), not the same problems' for the other kinds.
+constexpr uint32_t kAllKinds = (1u << K_NKINDS) - 1u;
+constexpr uint32_t kAlignedPatchKinds = (1u << K_COPY) | (1u << K_AXPBY2);  // f64; c64: all
+constexpr int64_t kL2Bytes = int64_t(126) << 20;
+
+uint32_t take_patches(const Plan &plan, std::vector<TileDesc> &list, PatchList &out, bool &rest) {
     static const int mode = [] {
         const char *e = std::getenv("COSTA_PATCH");
         return e ? std::atoi(e) : -1;
     }();
-    if (mode == 0 || list.empty()) return;
+    rest = true;
+    if (mode == 0 || list.empty()) return 0;
     const int es = plan.esize;
-    int64_t all = 0, poor = 0;
+    const bool cplx = plan.dtype == COSTA_C64 || plan.dtype == COSTA_C128;
+    int64_t all = 0, poor = 0, mis = 0, runs = 0, boxes = 0, small = 0;
+    for (const ProblemHost &ph : plan.probs) all += ph.A->m * ph.A->n;
+    const bool many = all >= 3000000;
     for (const TileDesc &d : list) {
         const int64_t e = static_cast<int64_t>(d.nx) * d.ny;
-        all += e;
         const bool misaligned = es == 4 ? !aligned16(d.dst, static_cast<int64_t>(d.dld) * es) || d.nx % 4 != 0
                                         : !(d.flags & TF_FAST);
-        if (misaligned || is_small(d, es)) poor += e;
+        const bool tr = (d.flags & TF_TRANSPOSE) != 0;
+        const bool run = d.nx == d.dld;  // one contiguous run of A
+        const bool sm = is_small(d, es);
+        // in large lists, 4- and 8-byte tiles along A's runs are poor below 16 x 16 only
+        const bool along = many && !tr && es < 16 && d.nx >= 16 && d.ny >= 16;
+        const bool partial = es != 4 && 4 * e < 3 * int64_t(plan.ts) * plan.ts && !run;
+        if (misaligned || (!along && (partial || sm))) poor += e;
+        if (misaligned) mis += e;
+        if (sm) small += e;
+        if (run) runs += e;
+        const int nr = tr ? d.nx : d.ny, len = tr ? d.ny : d.nx;
+        if (!misaligned && (nr == 16 || nr == 32) && len * es % 128 == 0) boxes += e;  // could be staged by TMA
     }
-    if (2 * poor < all && mode != 1) return;
-    std::vector<char> taken(plan.probs.size(), 0);
-    bool any = false;
-    for (size_t k = 0; k < taken.size(); ++k)
-        any |= (taken[k] = append_patches(plan.probs[k], static_cast<int>(k), out)) != 0;
-    if (!any) return;
-    size_t w = 0;
-    for (const TileDesc &d : list)
-        if (!taken[d.prob]) list[w++] = d;
-    list.resize(w);
+    const size_t n = plan.probs.size();
+    if (2 * poor >= all || (es == 8 && 20 * mis >= all) || mode == 1) {
+        std::vector<char> taken(n, 0);
+        bool any = false;
+        for (size_t k = 0; k < n; ++k)
+            any |= (taken[k] = append_patches(plan.probs[k], static_cast<int>(k), all, out)) != 0;
+        if (!any) return 0;
+        size_t w = 0;
+        for (const TileDesc &d : list)
+            if (!taken[d.prob]) list[w++] = d;
+        list.resize(w);
+        return kAllKinds;
+    }
+    if (es != 8 || 2 * all * es <= kL2Bytes || 2 * runs >= all || 4 * small >= all || tma_mode() == 1) return 0;
+    for (size_t k = 0; k < n; ++k)
+        if (!append_patches(plan.probs[k], static_cast<int>(k), all, out)) {
+            out.patches.clear();
+            out.cells.clear();
+            return 0;
+        }
+    if (cplx || mis > 0) {
+        list.clear();
+        return kAllKinds;
+    }
+    rest = false;
+    return kAlignedPatchKinds | (4 * boxes < 3 * all ? 1u << K_AXPBY : 0u);
 }
 
 // Builds the overlay, the tile list and the device tables, and runs the
@@ -477,12 +538,13 @@ costa_status build_plan(int n, const costa_layout *As, const costa_layout *Bs, c
     }
     const bool cplx = plan->dtype == COSTA_C64 || plan->dtype == COSTA_C128;
     PatchList patches;
-    take_patches(*plan, list, patches);
+    bool rest = true;
+    const uint32_t patch_kinds = take_patches(*plan, list, patches, rest);
     SplitList split = split_small(std::move(list), es, cplx);
     // The aligned tiles also as x-halves (see use_halves), for the kinds
     // that run on them (see launch_list in transform_impl).
     std::vector<char> halve(static_cast<size_t>(n), 0);
-    for (int k = 0; k < n; ++k) halve[k] = use_halves(plan->probs[k], es);
+    for (int k = 0; k < n; ++k) halve[k] = rest && use_halves(plan->probs[k], es);
     std::vector<TileDesc> halves = split_x_halves(split.big, ts / 2, es, halve);
     const bool had_halves = !halves.empty();
     // TMA staging (tma.cpp): the kinds the policy would give it; their lists
@@ -532,6 +594,8 @@ costa_status build_plan(int n, const costa_layout *As, const costa_layout *Bs, c
     plan->direct.patches = reinterpret_cast<const PatchDesc *>(dbase + off_patches);
     plan->direct.cells = reinterpret_cast<const PatchCell *>(dbase + off_pcells);
     plan->direct.npatches = static_cast<int64_t>(patches.patches.size());
+    plan->direct.patch_kinds = patch_kinds;
+    plan->direct.tiles_are_rest = rest;
     plan->direct_halves = plan->direct;
     if (had_halves) {
         plan->direct_halves.tiles = reinterpret_cast<const TileDesc *>(dbase + off_halves);
@@ -1115,9 +1179,10 @@ cudaError_t launch_split(const RemapLaunch &base, const DevList &list, const Dev
             lk.groups = list.groups_a;
             lk.ngroups = list.ngroups_a;
         }
-        cudaError_t e = launch_remap(lk, kind, stream);
+        const bool patches = list.npatches > 0 && ((list.patch_kinds >> kind) & 1u);
+        cudaError_t e = !patches || list.tiles_are_rest ? launch_remap(lk, kind, stream) : cudaSuccess;
         if (e != cudaSuccess) return e;
-        if (list.npatches > 0) {
+        if (patches) {
             PatchLaunch p{};
             p.patches = list.patches;
             p.cells = list.cells;
@@ -1515,7 +1580,7 @@ costa_status costa_debug_patches(costa_layout A, costa_layout B, costa_op op, vo
     ph.B = B;
     ph.op = op;
     PatchList l;
-    append_patches(ph, 0, l);
+    append_patches(ph, 0, A->m * A->n, l);
     *npatches = static_cast<int64_t>(l.patches.size());
     *ncells = static_cast<int64_t>(l.cells.size());
     const size_t kp = static_cast<size_t>(std::min<int64_t>(cap_patches, *npatches));

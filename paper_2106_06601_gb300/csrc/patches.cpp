@@ -238,7 +238,7 @@ bool one_order(const costa_layout_s *L, int &order) {
 
 }  // namespace
 
-bool append_patches(const ProblemHost &ph, int prob, PatchList &out) {
+bool append_patches(const ProblemHost &ph, int prob, int64_t total, PatchList &out) {
     const costa_layout_s *A = ph.A, *B = ph.B;
     int oa = 0, ob = 0;
     if (!one_order(A, oa) || !one_order(B, ob)) return false;
@@ -246,7 +246,19 @@ bool append_patches(const ProblemHost &ph, int prob, PatchList &out) {
     const bool op_tr = ph.op != COSTA_OP_N;
     const bool a_col = oa == COSTA_COL_MAJOR, b_col = ob == COSTA_COL_MAJOR;
     const bool transpose = a_col != (op_tr ? !b_col : b_col);
-    const int ex = patch_x(es), ey = patch_y(es);
+    int ex = patch_x(es), ey = patch_y(es);
+    // Few patches: smaller ones, with fewer passes along the run axis (and, for
+    // very few 8-byte ones, shorter runs), so that more warps share the work.
+    // us per call on GB300, whole / half / quarter patches:
+    //   f64 BC8 T beta = 0.5    512^2 5.2 / 3.7 / 3.5, 768^2 5.3 / 4.1 / 4.3,
+    //                           1024^2 5.8 / 5.2 / 6.7, 1536^2 12.3 / 13.2
+    //   f32 BC8 T beta = 0.5    512^2 3.1 / 2.8 / 3.1, 768^2 3.2 / 3.0 / 3.8,
+    //                           1024^2 3.6 / 3.8
+    //   c128 BC8 T beta = 0.5   256^2 3.6 / 3.0, 512^2 4.0 / 3.9, 768^2 5.4 / 6.1
+    int &run_ext = transpose ? ex : ey;
+    const int64_t half_below = es == 16 ? 300000 : es == 8 ? 1200000 : 700000;
+    if (total < half_below) run_ext /= 2;
+    if (es == 8 && total < 350000) (transpose ? ey : ex) /= 2;
     const int unit = std::max(1, std::min(ex, 128 / es));
     const AxisPatches rows = cut_patches(A, B, ph.op, 0, a_col ? ex : ey, a_col ? unit : 1);
     const AxisPatches cols = cut_patches(A, B, ph.op, 1, a_col ? ey : ex, a_col ? 1 : unit);

@@ -35,6 +35,8 @@ struct DevList {
     const PatchDesc *patches = nullptr;
     const PatchCell *cells = nullptr;
     int64_t npatches = 0;
+    uint32_t patch_kinds = 0;    // the kinds that run on the patches (bit per K_*)
+    bool tiles_are_rest = true;  // they also run on the tiles (other problems)
     bool empty() const { return ntiles == 0 && nmtiles == 0 && ngroups == 0 && npatches == 0; }
 };
 

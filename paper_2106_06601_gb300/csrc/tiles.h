@@ -137,13 +137,13 @@ std::vector<TileDesc> split_x_halves(const std::vector<TileDesc> &list, int hx, 
 // kind runs on the halves, and the f64 / c64 axpby kind with beta = +-2^k.
 bool use_halves(const ProblemHost &ph, int es);
 
-// The patches of problem `prob` (patches.cpp), appended to `out`; false (and
-// nothing appended) when its layouts mix element orders or need more cells
-// than a patch can index.
+// The patches of problem `prob` (patches.cpp) of a list of `total` elements,
+// appended to `out`; false (and nothing appended) when its layouts mix element
+// orders or need more cells than a patch can index.
 struct PatchList {
     std::vector<PatchDesc> patches;
     std::vector<PatchCell> cells;
 };
-bool append_patches(const ProblemHost &ph, int prob, PatchList &out);
+bool append_patches(const ProblemHost &ph, int prob, int64_t total, PatchList &out);
 
 }  // namespace costa

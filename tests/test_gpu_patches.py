@@ -42,6 +42,17 @@ def test_edges_of_patches(dtype, op, dev):
             check_problem(p, dev, guard=2)
 
 
+@pytest.mark.parametrize("dtype", ["f32", "f64", "c64", "c128"])
+@pytest.mark.parametrize("m, n", [(590, 601), (850, 870), (1101, 1107)])
+def test_extents_by_size(dtype, m, n, dev):
+    """The patch extents of each size class, with and without A."""
+    for op, (alpha, beta) in (("T", (1.0, 0.0)), ("N", (-0.3, 0.7)), ("C", (2.0, 0.5))):
+        B = L.block_cyclic(*((m, n) if op == "N" else (n, m)), 50, 37, 2, 2, ld_pad=1)
+        A = L.block_cyclic(m, n, 75, 24, 2, 2)
+        check_problem(C.Problem("patch", dtype, op, alpha, beta, A, B, "uniform", "nan" if beta == 0 else "uniform",
+                                C.SEED0 + 13), dev)
+
+
 def _special_doubles(n, rng):
     """Random doubles with all exponents, exact halfway products, zeros,
     subnormals, infinities and NaNs among runs of ordinary values."""

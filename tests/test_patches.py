@@ -109,9 +109,19 @@ def test_block_cyclic_forms(dtype, op, storage):
 def test_joined_blocks_make_few_cells():
     """On 1 x 1 grids every block continues its neighbours in storage, so a
     whole patch is one cell whatever the block sizes."""
-    B = L.block_cyclic(128, 96, 5, 7, 1, 1, name="B")
-    A = L.block_cyclic(96, 128, 3, 4, 1, 1, name="A")
+    B = L.block_cyclic(1280, 960, 5, 7, 1, 1, name="B")
+    A = L.block_cyclic(960, 1280, 3, 4, 1, 1, name="A")
     LA, LB = _layout(A, "f64"), _layout(B, "f64")
     patches, cells = costa.costa_debug_patches(LA, LB, "T")
-    assert len(patches) == 3 * 4 and len(cells) == len(patches)
+    assert len(patches) == 30 * 40 and len(cells) == len(patches)
     assert np.all(patches["nx"] == 32) and np.all(patches["ny"] == 32)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f64", "c128"])
+@pytest.mark.parametrize("m, n", [(590, 590), (850, 850), (1101, 1103)])
+def test_extents_by_size(dtype, m, n):
+    """Patch extents follow the matrix size: every size class covers A once."""
+    for op in "NT":
+        B = L.block_cyclic(*((m, n) if op == "N" else (n, m)), 50, 37, 2, 2, ld_pad=1, name="B")
+        A = L.block_cyclic(m, n, 75, 24, 2, 2, name="A")
+        assert check(C.Problem("patch", dtype, op, 1.0, 0.0, A, B))
