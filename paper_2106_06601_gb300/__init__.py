@@ -143,6 +143,33 @@ def _p(a: np.ndarray) -> int:
     return a.ctypes.data
 
 
+# Host arrays of the calls that run per transform are ctypes arrays made from
+# the caller's lists: 0.1 to 0.8 us each on the Grace host, where a numpy
+# conversion and the array's address take 1.1 to 2 (the GPU's work is often
+# shorter than that).
+_DESC = ctypes.c_int64 * 9
+
+
+def _desc(desc):
+    """A ScaLAPACK array descriptor as a C array (anything but a list of nine
+    integers goes through numpy)."""
+    if isinstance(desc, (list, tuple)) and len(desc) == 9:
+        try:
+            return _DESC(*desc)
+        except TypeError:
+            pass
+    return _i64(desc).ctypes
+
+
+def _sigma_out(nranks: int, relabel: int):
+    """(array, its memory) for a call's relabeling; without relabeling it is the
+    identity and the call need not write it."""
+    if not relabel:
+        return np.arange(nranks, dtype=np.int32), None
+    out = (ctypes.c_int32 * nranks)()
+    return np.frombuffer(out, dtype=np.int32), out
+
+
 class Layout:
     """Owning handle of a costa_layout."""
 
@@ -397,19 +424,16 @@ def costa_layout_create_scalapack(dtype: str, grid: BlacsGrid, i: int, j: int, m
 def costa_pxgemr2d(dtype: str, m: int, n: int, ga: BlacsGrid, ia: int, ja: int, desca,
                    gb: BlacsGrid, ib: int, jb: int, descb, stream: int = 0) -> None:
     """sub(B) := sub(A) (ScaLAPACK PxGEMR2D; 1-based ia, ja, ib, jb)."""
-    da, db = _i64(desca), _i64(descb)
-    _check(_lib.costa_pxgemr2d(DTYPES[dtype], m, n, ga.ref(), ia, ja, _p(da), gb.ref(), ib, jb,
-                               _p(db), ctypes.c_void_p(stream)))
+    _check(_lib.costa_pxgemr2d(DTYPES[dtype], m, n, ga.ref(), ia, ja, _desc(desca), gb.ref(), ib, jb,
+                               _desc(descb), stream))
 
 
 def costa_pxtran(dtype: str, m: int, n: int, alpha, ga: BlacsGrid, ia: int, ja: int, desca, beta,
                  gc: BlacsGrid, ic: int, jc: int, descc, conjugate: bool = False,
                  stream: int = 0) -> None:
     """sub(C) := beta sub(C) + alpha op(sub(A)), op = T (PxTRAN) or C (PxTRANC)."""
-    da, dc = _i64(desca), _i64(descc)
-    al, be = _scalars(dtype, [alpha]), _scalars(dtype, [beta])
-    _check(_lib.costa_pxtran(DTYPES[dtype], int(conjugate), m, n, _p(al), ga.ref(), ia, ja,
-                             _p(da), _p(be), gc.ref(), ic, jc, _p(dc), ctypes.c_void_p(stream)))
+    _check(_lib.costa_pxtran(DTYPES[dtype], int(conjugate), m, n, _scalar_arg(dtype, alpha), ga.ref(), ia, ja,
+                             _desc(desca), _scalar_arg(dtype, beta), gc.ref(), ic, jc, _desc(descc), stream))
 
 
 def costa_scalapack_release() -> None:
@@ -474,28 +498,48 @@ def _scalar1(dtype: str, v):
     return _SCALAR_CT[dtype](v.real, v.imag)
 
 
+def _scalar_arg(dtype: str, v):
+    """A host scalar as a pointer argument (array-likes go through numpy)."""
+    try:
+        return ctypes.byref(_scalar1(dtype, v))
+    except TypeError:
+        return _scalars(dtype, [v]).ctypes
+
+
+def _scalar_list(dtype: str, values, n: int):
+    """n host scalars as a pointer argument."""
+    if dtype in ("f32", "f64") and isinstance(values, (list, tuple)) and len(values) == n:
+        try:
+            return (_SCALAR_CT[dtype] * n)(*values)
+        except TypeError:
+            pass
+    a = _scalars(dtype, values)
+    assert a.size == n
+    return a.ctypes
+
+
 def costa_transform(A: Layout, B: Layout, op: str, alpha, beta, relabel: bool = False,
                     stream: int = 0, mode: str = "direct") -> np.ndarray:
     """A = alpha * op(B) + beta * A, asynchronous on `stream`; returns sigma."""
-    sigma = np.zeros(A.nranks, dtype=np.int32)
+    relabel = int(relabel)
+    sigma, out = _sigma_out(A.nranks, relabel)
     al, be = _scalar1(A.dtype, alpha), _scalar1(A.dtype, beta)
     _check(_lib.costa_transform_ex(A.handle, B.handle, OPS[op], ctypes.byref(al), ctypes.byref(be),
-                                   int(relabel), sigma.ctypes.data, MODES[mode], stream))
+                                   relabel, out, MODES[mode], stream))
     return sigma
 
 
 def costa_transform_batched(As, Bs, ops, alphas, betas, relabel: bool = False,
                             stream: int = 0, mode: str = "direct") -> np.ndarray:
     n = len(As)
-    _, _, P, _ = As[0].info()
-    sigma = np.zeros(P, dtype=np.int32)
-    ha = (ctypes.c_void_p * n)(*[a.handle.value for a in As])
-    hb = (ctypes.c_void_p * n)(*[b.handle.value for b in Bs])
-    op = _i32([OPS[o] for o in ops])
-    al, be = _scalars(As[0].dtype, alphas), _scalars(As[0].dtype, betas)
-    assert al.size == n and be.size == n
-    _check(_lib.costa_transform_batched_ex(n, ha, hb, _p(op), _p(al), _p(be), int(relabel),
-                                           _p(sigma), MODES[mode], ctypes.c_void_p(stream)))
+    relabel = int(relabel)
+    sigma, out = _sigma_out(As[0].nranks, relabel)
+    handles = ctypes.c_void_p * n
+    ha = handles(*[a.handle.value for a in As])
+    hb = handles(*[b.handle.value for b in Bs])
+    op = (ctypes.c_int32 * n)(*[OPS[o] for o in ops])
+    al, be = _scalar_list(As[0].dtype, alphas, n), _scalar_list(As[0].dtype, betas, n)
+    _check(_lib.costa_transform_batched_ex(n, ha, hb, op, al, be, relabel, out, MODES[mode], stream))
     return sigma
 
 

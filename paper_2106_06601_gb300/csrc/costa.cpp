@@ -516,7 +516,7 @@ costa_status build_plan(int n, const costa_layout *As, const costa_layout *Bs, c
     // the direct tile list, in (problem, row piece, column piece) order
     std::vector<TileDesc> list;
     if (n == 1) {
-        append_direct_tiles(plan->probs[0], 0, es, ts, list);
+        append_direct_tiles(plan->probs[0], 0, es, ts, list, false);  // ordered below, if the tiles are kept
     } else {  // a batch: problems in parallel, each into its own range
         std::vector<int64_t> start(static_cast<size_t>(n) + 1, 0);
         for (int k = 0; k < n; ++k)
@@ -540,6 +540,7 @@ costa_status build_plan(int n, const costa_layout *As, const costa_layout *Bs, c
     PatchList patches;
     bool rest = true;
     const uint32_t patch_kinds = take_patches(*plan, list, patches, rest);
+    if (n == 1) order_direct_tiles(plan->probs[0], list, 0, es, ts);
     SplitList split = split_small(std::move(list), es, cplx);
     // The aligned tiles also as x-halves (see use_halves), for the kinds
     // that run on them (see launch_list in transform_impl).
@@ -863,7 +864,8 @@ costa_status get_plan(int n, const costa_layout *A, const costa_layout *B, const
     int dev = 0;
     cudaError_t ce = cudaGetDevice(&dev);
     if (ce != cudaSuccess) return cuda_fail(ce, "cudaGetDevice");
-    std::vector<uint64_t> key;
+    static thread_local std::vector<uint64_t> key;  // keeps its storage between calls
+    key.clear();
     key.reserve(2 + 3 * static_cast<size_t>(n));
     key.push_back(static_cast<uint64_t>(dev));
     key.push_back(static_cast<uint64_t>(n));
@@ -881,7 +883,7 @@ costa_status get_plan(int n, const costa_layout *A, const costa_layout *B, const
     costa_status s = build_plan(n, A, B, ops, stream, plan);
     if (s != COSTA_OK) return s;
     out = plan.get();
-    g_plans.emplace(std::move(key), std::move(plan));
+    g_plans.emplace(key, std::move(plan));
     return COSTA_OK;
 }
 
@@ -931,14 +933,19 @@ costa_status transform_impl(int n, const costa_layout *A, const costa_layout *B,
     L.s = make_scalars(plan->dtype, alphas, betas, 0);
     L.per_problem = nullptr;
     bool uniform = true;
-    std::vector<Scalars> sc(n);
-    for (int k = 0; k < n; ++k) {
-        sc[k] = make_scalars(plan->dtype, alphas, betas, k);
-        if (!same_scalars(sc[k], sc[0])) uniform = false;
-    }
+    std::vector<Scalars> sc;  // a batch's scalars
     // one launch per combine kind present in the batch
     bool kinds[K_NKINDS] = {};
-    for (int k = 0; k < n; ++k) kinds[kind_of(sc[k].flags)] = true;
+    kinds[kind_of(L.s.flags)] = true;
+    if (n > 1) {
+        sc.resize(static_cast<size_t>(n));
+        sc[0] = L.s;
+        for (int k = 1; k < n; ++k) {
+            sc[k] = make_scalars(plan->dtype, alphas, betas, k);
+            if (!same_scalars(sc[k], sc[0])) uniform = false;
+            kinds[kind_of(sc[k].flags)] = true;
+        }
+    }
     if (!plan->tma_built && mode == COSTA_MODE_DIRECT) {
         bool want = false;
         for (int kind = 0; kind < K_NKINDS; ++kind)

@@ -469,8 +469,19 @@ void order_tiles_local(std::vector<TileDesc> &list, size_t first, size_t last, i
     std::copy(tmp.begin(), tmp.end(), list.begin() + static_cast<std::ptrdiff_t>(first));
 }
 
-// Appends the direct tiles of problem `prob` in the kernel's order.
-void append_direct_tiles(const ProblemHost &ph, int prob, int es, int ts, std::vector<TileDesc> &list) {
+// Puts the tiles [first, end) of one problem, appended in the global order,
+// into the kernel's order.
+void order_direct_tiles(const ProblemHost &ph, std::vector<TileDesc> &list, size_t first, int es, int ts) {
+    if (!use_local_order(ph, list.data() + first, list.size() - first)) return;
+    // a target whose tiles are each one contiguous run gains nothing
+    bool contiguous = true;
+    for (size_t i = first; i < list.size() && contiguous; ++i) contiguous = list[i].nx == list[i].dld;
+    if (!contiguous) order_tiles_local(list, first, list.size(), es, ts);
+}
+
+// Appends the direct tiles of problem `prob` in the kernel's order, or in the
+// global super-tile order for a later order_direct_tiles.
+void append_direct_tiles(const ProblemHost &ph, int prob, int es, int ts, std::vector<TileDesc> &list, bool ordered) {
     const size_t first = list.size();
     // the order of for_each_tile, built in parallel over bands of kSuper row
     // pieces: band su holds the tiles [su * nv, (su + band rows) * nv)
@@ -492,11 +503,7 @@ void append_direct_tiles(const ProblemHost &ph, int prob, int es, int ts, std::v
                     }
         }
     });
-    if (!use_local_order(ph, list.data() + first, list.size() - first)) return;
-    // a target whose tiles are each one contiguous run gains nothing
-    bool contiguous = true;
-    for (size_t i = first; i < list.size() && contiguous; ++i) contiguous = list[i].nx == list[i].dld;
-    if (!contiguous) order_tiles_local(list, first, list.size(), es, ts);
+    if (ordered) order_direct_tiles(ph, list, first, es, ts);
 }
 
 }  // namespace costa

@@ -114,7 +114,9 @@ bool mostly_misaligned(const TileDesc *tiles, size_t n, int es, bool target_only
 bool use_local_order(const ProblemHost &ph, const TileDesc *tiles, size_t n);
 void radix_sort_pairs(std::vector<std::pair<uint64_t, uint32_t>> &v);
 void order_tiles_local(std::vector<TileDesc> &list, size_t first, size_t last, int es, int ts);
-void append_direct_tiles(const ProblemHost &ph, int prob, int es, int ts, std::vector<TileDesc> &list);
+void order_direct_tiles(const ProblemHost &ph, std::vector<TileDesc> &list, size_t first, int es, int ts);
+void append_direct_tiles(const ProblemHost &ph, int prob, int es, int ts, std::vector<TileDesc> &list,
+                         bool ordered = true);
 
 int next_pow2(int v);
 int fast_tile_passes(const TileDesc &d, int es);
