@@ -343,7 +343,9 @@ __global__ void __launch_bounds__(PCfg<T, KIND>::WARPS * 32, PCfg<T, KIND>::MINB
             return;
         }
     };
+    if (args.per_problem) pdl_wait();  // advance reads the batch's scalars
     advance();
+    pdl_wait();
     while (more) {
         const PatchDesc d = next;
         put_cells(cr, cells, lane);
@@ -379,9 +381,9 @@ cudaError_t launch_patch(const PatchLaunch &a, cudaStream_t st) {
     const int64_t cap = static_cast<int64_t>(sm_count()) * per_sm;
     const int blocks = static_cast<int>(want < cap ? want : cap);
     if (blocks <= 0) return cudaSuccess;
-    kern<<<blocks, P::WARPS * 32, smem, st>>>(a);
-    count_launch();
-    return cudaGetLastError();
+    const cudaError_t e = pdl_launch(kern, blocks, P::WARPS * 32, smem, st, a);
+    if (e == cudaSuccess) count_launch();
+    return e;
 }
 
 template <typename T>
