@@ -548,6 +548,8 @@ costa_status build_plan(int n, const costa_layout *As, const costa_layout *Bs, c
     for (int k = 0; k < n; ++k) halve[k] = rest && use_halves(plan->probs[k], es);
     std::vector<TileDesc> halves = split_x_halves(split.big, ts / 2, es, halve);
     const bool had_halves = !halves.empty();
+    split.big = cut_few(std::move(split.big), es);
+    halves = cut_few(std::move(halves), es);
     // TMA staging (tma.cpp): the kinds the policy would give it; their lists
     // are built by the first call of such a kind (ensure_tma)
     plan->tma_kinds_big = tma_policy_kinds(split.big, es, cplx, false);

@@ -469,6 +469,25 @@ void order_tiles_local(std::vector<TileDesc> &list, size_t first, size_t last, i
     std::copy(tmp.begin(), tmp.end(), list.begin() + static_cast<std::ptrdiff_t>(first));
 }
 
+std::vector<TileDesc> cut_few(std::vector<TileDesc> &&list, int es) {
+    int parts = 1;
+    while (parts < 4 && list.size() * parts * 2 <= few_tiles(es)) parts *= 2;
+    if (parts == 1 || list.empty()) return std::move(list);
+    std::vector<TileDesc> out;
+    out.reserve(list.size() * parts);
+    for (const TileDesc &t : list) {
+        const int rows = ((t.ny + parts - 1) / parts + 3) / 4 * 4;  // whole 16-byte chunks of every type
+        for (int y = 0; y < t.ny; y += rows) {
+            TileDesc d = t;
+            d.dst += static_cast<uint64_t>(static_cast<int64_t>(y) * t.dld * es);
+            d.src += static_cast<uint64_t>(((t.flags & TF_TRANSPOSE) ? y : static_cast<int64_t>(y) * t.sld) * es);
+            d.ny = static_cast<uint16_t>(std::min<int>(rows, t.ny - y));
+            out.push_back(d);
+        }
+    }
+    return out;
+}
+
 // Puts the tiles [first, end) of one problem, appended in the global order,
 // into the kernel's order.
 void order_direct_tiles(const ProblemHost &ph, std::vector<TileDesc> &list, size_t first, int es, int ts) {

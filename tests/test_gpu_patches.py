@@ -53,6 +53,18 @@ def test_extents_by_size(dtype, m, n, dev):
                                 C.SEED0 + 13), dev)
 
 
+@pytest.mark.parametrize("dtype", ["f32", "f64", "c64", "c128"])
+@pytest.mark.parametrize("m, n", [(32, 64), (68, 36), (128, 128), (600, 404), (800, 768)])
+def test_lists_of_few_tiles(dtype, m, n, dev):
+    """Short lists of aligned tiles, which are cut into halves and quarters
+    by rows: one tile, ragged tiles, and lists about the limit."""
+    for op, (alpha, beta) in zip("TNCT", KINDS.values()):
+        B = L.block_cyclic(*((m, n) if op == "N" else (n, m)), 64, 32, 1, 2)
+        A = L.block_cyclic(m, n, 32, 128, 2, 1)
+        check_problem(C.Problem("few", dtype, op, alpha, beta, A, B, "uniform", "nan" if beta == 0 else "uniform",
+                                C.SEED0 + 15), dev, guard=4)
+
+
 def _special_doubles(n, rng):
     """Random doubles with all exponents, exact halfway products, zeros,
     subnormals, infinities and NaNs among runs of ordinary values."""
