@@ -101,7 +101,7 @@ struct PatchDesc {
     uint32_t lmask, rmask;
     uint8_t nx, ny;  // extents
     uint16_t prob;   // problem index within the launch
-    uint16_t flags;  // TF_TRANSPOSE, TF_CONJ
+    uint16_t flags;  // TF_TRANSPOSE, TF_CONJ; TF_FAST: 4-byte patches staged by 16-byte chunks
     uint16_t pad;
 };
 static_assert(sizeof(PatchDesc) == 32, "PatchDesc layout");

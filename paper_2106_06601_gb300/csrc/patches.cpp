@@ -330,8 +330,10 @@ bool append_patches(const ProblemHost &ph, int prob, int64_t total, PatchList &o
                 d.prob = static_cast<uint16_t>(prob);
                 d.flags = static_cast<uint16_t>((transpose ? TF_TRANSPOSE : 0) | (ph.op == COSTA_OP_C ? TF_CONJ : 0));
                 d.pad = 0;
-                out.patches[static_cast<size_t>(row.patch0) + (x - row.x0)] = d;
                 const AxisPatch &run = transpose ? px : py, &lane = transpose ? py : px;
+                // 4-byte elements: source runs of whole aligned 16-byte chunks, and
+                // one row of A per pass
+                bool chunks = es == 4 && d.nx > 16 && lane.len % 4 == 0 && (lane.mask & 0xEEEEEEEEu) == 0;
                 const std::vector<PatchSeg> &rs = transpose ? X.segs : Y.segs, &ls = transpose ? Y.segs : X.segs;
                 for (int r = 0; r < run.nseg; ++r)
                     for (int l = 0; l < lane.nseg; ++l) {
@@ -347,8 +349,11 @@ bool append_patches(const ProblemHost &ph, int prob, int64_t total, PatchList &o
                         c.src = db.ptr + static_cast<uint64_t>((off - sr.start * static_cast<int64_t>(db.ld) - sl.start) * es);
                         c.sld = db.ld;
                         c.pad = 0;
+                        chunks = chunks && c.src % 16 == 0 && db.ld % 4 == 0;
                         out.cells[static_cast<size_t>(cell++)] = c;
                     }
+                if (chunks) d.flags = static_cast<uint16_t>(d.flags | TF_FAST);
+                out.patches[static_cast<size_t>(row.patch0) + (x - row.x0)] = d;
             }
         }
     });

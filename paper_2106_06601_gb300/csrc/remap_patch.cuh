@@ -40,8 +40,8 @@ namespace remap {
 //   f64 copy  175   161   171   167   190   (BC8)
 //   f64 b=0.5 327   262   242   243   393   (BC8)
 //   f64 scale  -    211   206   218    -    (BC50 -> BC75)
-//   f32 copy  130   109   104   102   101   (BC8)
-//   f32 b=0.5 177   149   139   156   165   (BC8)
+//   f32 copy   -     -     89    84    91   (BC8)
+//   f32 b=0.5 177   149   130   197    -    (BC8)
 //   c128 copy 248   200   179   178   192   (BC8)
 //   c128 b=.5 400   307   267   269   470   (BC8)
 #ifndef COSTA_PW
@@ -85,13 +85,16 @@ template <typename T, int KIND> struct PCfg {
     static constexpr int EX = patch_x(ES), EY = patch_y(ES);
     // staged rows, one run of the source each: an odd pitch, so that lanes
     // reading one position of consecutive rows hit distinct banks
-    static constexpr int PITCH_T = EY + 1, PITCH_N = EX + 1;
+    static constexpr int PITCH_T = EY + 1, PITCH_N = ES == 4 ? EX + 4 : EX + 1;
     static constexpr int WARPS = COSTA_PW;
     static constexpr bool READS_A = kind_reads_a(KIND);
     // real doubles: part of the products beta * a and alpha * b are formed on
     // the integer pipes (mul_group)
     static constexpr bool INT_MUL = sizeof(T) == 8 && !ET<T>::CPLX;
     static constexpr int MINB = patch_blocks(ES, ET<T>::CPLX != 0, KIND);
+    // 4-byte elements: patches with TF_FAST stage whole 16-byte chunks (N: the
+    // pitch is whole chunks; T: rows of 128 bytes, chunk_slot)
+    static constexpr bool CHUNKED = ES == 4;
     static constexpr int ELEMS = EX * PITCH_T > EY * PITCH_N ? EX * PITCH_T : EY * PITCH_N;
     static constexpr int BUF = (ELEMS * ES + 15) / 16 * 16;
     static constexpr int CELLS = kPatchCells * 16;
@@ -153,16 +156,37 @@ __device__ __forceinline__ void put_cells(const CellRegs &c, uint4 *sm, int lane
     sm[lane + 32] = c.b;
 }
 
-// Copies a patch's source into `buf`, one run of the source per row.
+// Byte offset of chunk c of row r of a transposed patch that is staged by
+// 16-byte chunks: lanes that read chunk c of consecutive rows hit distinct banks.
+__device__ __forceinline__ int chunk_slot(int r, int c) { return r * 128 + ((c ^ (r & 7)) << 4); }
+
+// Copies a patch's source into `buf`, one run of the source per row.  4-byte
+// patches more than 16 elements wide whose source runs are whole aligned
+// 16-byte chunks (TF_FAST) copy those: they bypass the L1 and take a quarter of the instructions.  GB300,
+// 8192^2 f32 T, us per call, elements -> chunks: copy BC8 101 -> 84, A's ld odd
+// 109 -> 90; beta = 0.5 BC8 138 -> 130, A's ld odd 149 -> 134.
 template <typename T, int KIND>
 __device__ __forceinline__ void patch_stage(const PatchDesc &d, const uint4 *cells, unsigned char *buf, int lane) {
     using P = PCfg<T, KIND>;
     constexpr int ES = P::ES;
     const bool tr = (d.flags & TF_TRANSPOSE) != 0;
     const int nr = tr ? d.nx : d.ny, nl = tr ? d.ny : d.nx;
+    const int nls = __popc(d.lmask);
+    if (P::CHUNKED && (d.flags & TF_FAST)) {
+        const LaneMap m = lane_map(nl / 4, lane);
+        if (m.c >= nl / 4) return;
+        const uint4 *cl = cells + seg_of(d.lmask, m.c * 4);
+#pragma unroll 4
+        for (int r = m.r0; r < nr; r += m.rpp) {
+            const uint4 c = cl[seg_of(d.rmask, r) * nls];
+            const char *p = reinterpret_cast<const char *>((static_cast<uint64_t>(c.y) << 32) | c.x) + m.c * 16 +
+                            static_cast<int64_t>(r) * (static_cast<int64_t>(static_cast<int32_t>(c.z)) * 4);
+            cp_async16(buf + (tr ? chunk_slot(r, m.c) : r * (P::PITCH_N * 4) + m.c * 16), p);
+        }
+        return;
+    }
     const LaneMap m = lane_map(nl, lane);
     if (m.c >= nl) return;
-    const int nls = __popc(d.lmask);
     const uint4 *cl = cells + seg_of(d.lmask, m.c);
     const int pitch = tr ? P::PITCH_T : P::PITCH_N;
     unsigned char *sp = buf + (m.r0 * pitch + m.c) * ES;
@@ -218,8 +242,9 @@ __device__ __forceinline__ void mul_group(Chunk<T> (&v)[N], double c, unsigned m
     }
 }
 
-// Writes a staged patch to A in A's contiguous order, one element per lane.
-template <typename T, int KIND>
+// Writes a staged patch to A in A's contiguous order, one element per lane
+// (CHUNKS: a transposed patch that is staged by 16-byte chunks).
+template <typename T, int KIND, bool CHUNKS>
 __device__ __forceinline__ void patch_write(const PatchLaunch &a, const PatchDesc &d, Sc &s, int &cached,
                                             const unsigned char *buf, int lane) {
     using P = PCfg<T, KIND>;
@@ -229,7 +254,7 @@ __device__ __forceinline__ void patch_write(const PatchLaunch &a, const PatchDes
         cached = d.prob;
     }
     s.conj_mask = ET<T>::CPLX && (d.flags & TF_CONJ) ? 0x80000000u : 0u;
-    const bool tr = (d.flags & TF_TRANSPOSE) != 0;
+    const bool tr = CHUNKS || (d.flags & TF_TRANSPOSE) != 0;
     const LaneMap m = lane_map(d.nx, lane);
     const bool on = m.c < d.nx;
     const unsigned mask = __ballot_sync(0xffffffffu, on);
@@ -240,6 +265,13 @@ __device__ __forceinline__ void patch_write(const PatchLaunch &a, const PatchDes
     const int64_t step = static_cast<int64_t>(m.rpp) * d.dld;
     const unsigned char *sp = buf + (tr ? m.c * P::PITCH_T + m.r0 : m.r0 * P::PITCH_N + m.c) * ES;
     const int sstep = m.rpp * (tr ? ES : P::PITCH_N * ES);
+    // CHUNKS: the staged elements of rows p .. p + 3 (a pass is one row; p a
+    // multiple of 4)
+    auto staged4 = [&](int p) {
+        Chunk<T> b;
+        b.raw = *reinterpret_cast<const uint4 *>(buf + chunk_slot(m.c, p / 4));
+        return b;
+    };
     Chunk<T> av[2][NC];
     const T *q = dst;
     auto load = [&](Chunk<T> (&v)[NC], int p0) {  // A's elements of passes p0 .. p0 + G - 1
@@ -254,11 +286,27 @@ __device__ __forceinline__ void patch_write(const PatchLaunch &a, const PatchDes
     auto write = [&](Chunk<T> (&v)[NC], int p0) {
         if (KIND == K_AXPBY2) prescale<T>(v, NC, s, mask);
         if constexpr (KIND == K_AXPBY && P::INT_MUL) mul_group<T>(v, s.br, mask);  // beta * a, then as K_AXPBY2
+        if constexpr (CHUNKS) {
 #pragma unroll
-        for (int k = 0; k < G; ++k) {
-            if (p0 + k < cnt) *dst = combine<KIND == K_AXPBY && P::INT_MUL ? K_AXPBY2 : KIND>(*reinterpret_cast<const T *>(sp), v[k / V].e[k % V], s);
-            dst += step;
-            sp += sstep;
+            for (int c = 0; c < G; c += 4) {
+                if (p0 + c >= npass) break;  // uniform across the warp
+                const Chunk<T> b = staged4(p0 + c);
+#pragma unroll
+                for (int k = c; k < c + 4; ++k) {
+                    if (p0 + k < cnt) *dst = combine<KIND>(b.e[(k - c) % V], v[k / V].e[k % V], s);
+                    dst += step;
+                }
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < G; ++k) {
+                if (p0 + k < cnt) {
+                    const T b = *reinterpret_cast<const T *>(sp);
+                    *dst = combine<KIND == K_AXPBY && P::INT_MUL ? K_AXPBY2 : KIND>(b, v[k / V].e[k % V], s);
+                }
+                dst += step;
+                sp += sstep;
+            }
         }
     };
     if (P::READS_A && on) {
@@ -293,6 +341,16 @@ __device__ __forceinline__ void patch_write(const PatchLaunch &a, const PatchDes
 #pragma unroll
                 for (int k = 0; k < G; ++k) {
                     if (p0 + k < cnt) *dst = combine<K_COPY>(v[k / V].e[k % V], T(), s);
+                    dst += step;
+                }
+            }
+        } else if constexpr (CHUNKS) {
+#pragma unroll 2
+            for (int p = 0; p < npass; p += 4) {
+                const Chunk<T> b = staged4(p);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    if (p + k < cnt) *dst = combine<KIND>(b.e[k % V], T(), s);
                     dst += step;
                 }
             }
@@ -353,7 +411,13 @@ __global__ void __launch_bounds__(PCfg<T, KIND>::WARPS * 32, PCfg<T, KIND>::MINB
         advance();
         patch_stage<T, KIND>(d, cells, buf, lane);
         cp_async_commit();
-        patch_write<T, KIND>(args, d, s, cached, buf, lane);
+        if constexpr (P::CHUNKED) {
+            if ((d.flags & (TF_TRANSPOSE | TF_FAST)) == (TF_TRANSPOSE | TF_FAST)) {
+                patch_write<T, KIND, true>(args, d, s, cached, buf, lane);
+                continue;
+            }
+        }
+        patch_write<T, KIND, false>(args, d, s, cached, buf, lane);
     }
 }
 

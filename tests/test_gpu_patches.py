@@ -53,6 +53,19 @@ def test_extents_by_size(dtype, m, n, dev):
                                 C.SEED0 + 13), dev)
 
 
+@pytest.mark.parametrize("op", ["N", "T"])
+@pytest.mark.parametrize("mb, ma, pads", [(8, 16, (0, 0)), (8, 12, (4, 1)), (16, 5, (0, 0)), (24, 8, (8, 3))])
+def test_chunks_of_aligned_f32_runs(mb, ma, pads, op, dev):
+    """f32 patches that are staged by 16-byte chunks, beside ragged ones that
+    are not, for every kind."""
+    m, n = 1100, 1108
+    for alpha, beta in KINDS.values():
+        B = L.block_cyclic(*((m, n) if op == "N" else (n, m)), mb, mb, 2, 2, ld_pad=pads[0])
+        A = L.block_cyclic(m, n, ma, ma, 2, 2, ld_pad=pads[1])
+        check_problem(C.Problem("patch", "f32", op, alpha, beta, A, B, "uniform", "nan" if beta == 0 else "uniform",
+                                C.SEED0 + 14), dev)
+
+
 @pytest.mark.parametrize("dtype", ["f32", "f64", "c64", "c128"])
 @pytest.mark.parametrize("m, n", [(32, 64), (68, 36), (128, 128), (600, 404), (800, 768)])
 def test_lists_of_few_tiles(dtype, m, n, dev):

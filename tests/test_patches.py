@@ -49,6 +49,9 @@ def _patch_moves(patches, cells, es):
         k = rs[r] * nls + ls[l]
         # biased addresses wrap modulo 2^64
         s = (c["src"][k] + ((r * c["sld"].astype(np.int64)[k] + l) * es).astype(np.uint64)).astype(np.int64)
+        if p["flags"] & 2:  # staged by whole aligned 16-byte chunks
+            q = s.reshape(nr, nl // 4, 4)
+            assert es == 4 and nx > 16 and np.all(q[..., 0] % 16 == 0) and np.all(np.diff(q, axis=2) == 4)
         x, y = (r, l) if tr else (l, r)
         d = int(p["dst"]) + (x + y * int(p["dld"])) * es
         out.append(np.stack([d.ravel(), s.ravel()]))
@@ -125,3 +128,20 @@ def test_extents_by_size(dtype, m, n):
         B = L.block_cyclic(*((m, n) if op == "N" else (n, m)), 50, 37, 2, 2, ld_pad=1, name="B")
         A = L.block_cyclic(m, n, 75, 24, 2, 2, name="A")
         assert check(C.Problem("patch", dtype, op, 1.0, 0.0, A, B))
+
+
+@pytest.mark.parametrize("op", ["N", "T"])
+@pytest.mark.parametrize("mb, ma, pad, chunks", [(8, 16, 0, True), (64, 128, 0, True), (8, 12, 4, True), (64, 64, 1, False),
+                                                 (6, 16, 0, False)])
+def test_chunks_of_aligned_f32_runs(op, mb, ma, pad, chunks):
+    """f32 patches are staged by 16-byte chunks exactly where their source
+    runs allow it (checked patch by patch in _patch_moves)."""
+    m, n = 1100, 1108
+    B = L.block_cyclic(*((m, n) if op == "N" else (n, m)), mb, mb, 2, 2, ld_pad=pad, name="B")
+    A = L.block_cyclic(m, n, ma, ma, 2, 2, ld_pad=1, name="A")
+    p = C.Problem("patch", "f32", op, 1.0, 0.0, A, B)
+    assert check(p)
+    LA, LB = _layout(A, "f32"), _layout(B, "f32")
+    patches, _ = costa.costa_debug_patches(LA, LB, op)
+    share = np.mean((patches["flags"] & 2) != 0)
+    assert share > 0.5 if chunks else share < 0.25
