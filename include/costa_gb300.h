@@ -484,8 +484,9 @@ const char *costa_last_error(void);
 costa_status costa_debug_axis_pieces(costa_layout A, costa_layout B, costa_op op, int axis,
                                      int32_t *out, int64_t cap, int64_t *count);
 
-/* Diagnostics (host only, no device work): the remap kernel's tile list for
- * (A, B, op) in direct mode, in the order the kernel's warps take the tiles.  Each tile is 32 bytes: {source address, target
+/* Diagnostics (host only, no device work): the tile kernel's list for
+ * (A, B, op) in direct mode, in the order the kernel's warps take the tiles
+ * (pairs that run on patches move the same elements by those).  Each tile is 32 bytes: {source address, target
  * address (uint64), source stride, target stride (int32), nx, ny, problem,
  * flags (uint16)}, in the frame where x runs along A's contiguous axis
  * (flags: 1 = transposed, 2 = vector path, 4 = conjugate).  Writes
@@ -494,7 +495,8 @@ costa_status costa_debug_tiles(costa_layout A, costa_layout B, costa_op op, void
                                int64_t *count);
 
 /* Diagnostics (host only, no device work): how the direct tile list of
- * (A, B, op) is split between the two remap kernels.  Tiles needing fewer
+ * (A, B, op) is split between the tile kernel and the small-tile kernel, for
+ * pairs that do not run on patches (costa_debug_patches).  Tiles needing fewer
  * than half of a full tile's warp passes are cut into pieces of one warp
  * pass each (at most 8 x 8 elements; 16 x 8 for 4-byte and 8 x 4 for
  * 16-byte elements, x along A's contiguous axis), which the small-tile
@@ -521,7 +523,8 @@ costa_status costa_debug_groups(costa_layout A, costa_layout B, costa_op op, int
 
 /* Diagnostics (host only, no device work): the aligned full-size tiles of
  * (A, B, op) as x-halves, the list that the f32 kinds and the f64 / c64
- * axpby kind with beta = +-2^k run on.  A tile at least 32 high and wider
+ * axpby kind with beta = +-2^k run on (pairs that do not run on patches).  A
+ * tile at least 32 high and wider
  * than 16 along A's contiguous axis becomes two tiles, columns [0, 16) and
  * the rest, adjacent in the list; the others stay as they are.  Writes up
  * to cap_tiles 32-byte descriptors (as in costa_debug_tiles) to `tiles` and
@@ -543,13 +546,15 @@ costa_status costa_debug_exchange(costa_layout A, costa_layout B, costa_op op, i
 
 /* Diagnostics (host only, no device work): the patches of (A, B, op), the
  * work list of the patch kernel, which moves pairs whose overlay cells are
- * mostly small or misaligned.  A patch is a window of A's storage (at most
- * 32 x 32 elements; 16 x 16 for 16-byte elements) that may cover several
- * overlay cells: 32 bytes {target address (uint64), target stride (int32),
+ * mostly small, partial or misaligned, and large ones of 4- and 8-byte
+ * elements.  A patch is a window of A's storage (at most
+ * 32 x 32 elements, 16 x 16 for 16-byte elements; less for small matrices)
+ * that may cover several overlay cells: 32 bytes {target address (uint64), target stride (int32),
  * first cell (uint32), lmask, rmask (uint32), nx, ny (uint8), problem, flags,
  * padding (uint16)}, x along A's contiguous axis.  The source is cut into
  * segments along the lane axis (the source's contiguous one: y when flags
- * has 1 = transposed, else x) and the run axis (the other): bit k of lmask /
+ * has 1 = transposed, else x; 2: 4-byte source runs of whole aligned 16-byte
+ * chunks) and the run axis (the other): bit k of lmask /
  * rmask is set where one starts.  Segment pair (r, l) is cell first + r *
  * popcount(lmask) + l, 16 bytes {address (uint64), source stride (int32),
  * padding}: its element (run i, lane j of the patch) is at address +

@@ -393,27 +393,66 @@ costa_status check_access(costa_layout_s *L, int dev, const char *which) {
 //   BC16, T        f64 copy 182 -> 161; f32 copy 112 -> 101, beta = 0.5 146
 //                  -> 139; c128 beta = 0.5 375 -> 266
 // f32 with only B's ld odd: copy 99 -> 105 (kept on the window path).
+// Doubles in aligned cells whose extents are powers of two from 8 on keep the
+// kinds that read A on the tile kernels in lists of middle size, where a
+// patch kernel's two or three rounds of patches leave the last one half empty
+// (T, us, tiles / patches): beta = 0.5 BC8 1536^2 15.4 / 12.6, 1664^2 16.8 /
+// 17.1, 2816^2 35.3 / 36.9, BC16 -> BC32 4096^2 66.7 / 68.8, 5120^2 faster;
+// beta = 0.7 BC8 -> BC64 2048^2 25.3 / 26.6, 6144^2 154.9 / 162.6.  With op's
+// runs along A's and B's blocks the larger ones, lines of B are shared and the
+// line lies lower (BC64 -> BC8, N, beta = 0.5: 2816^2 37.9 / 38.5, 4096^2 1.23
+// times faster).  alpha = 1.5 with blocks of different sizes likewise (BC8 ->
+// BC64 2048^2 faster, 4096^2 50.2 / 52.4, 6144^2 104.7 / 108.0).  8-byte copies
+// of partial but not small tiles stay up to 1.75 times the L2 (BC48 2048^2 13.4
+// / 14.2, 2816^2 23.3 / 23.9, BC24 3072^2 26.6 / 27.5, BC48 4096^2 48.0 / 44.7),
+// and f32 copies of cells of 16 x 16 and more between blocks whose ratio is no
+// power of two (BC16 -> BC48 8064^2 99 / 117, beta = 0.5 142 / 140; BC16 -> BC32
+// faster), with A's blocks the smaller ones every kind (BC48 -> BC16 8192^2
+// beta = 0.5 142 / 144).
 //
-// 2. Aligned lists of 8-byte elements with more data than the L2 cache holds
-// and targets that are not one contiguous run per tile: the kinds in
-// kAlignedPatchKinds run on patches (if every problem has them), the other
-// f64 kinds on the tiles, unless some are misaligned (two or three launches: a
+// 2. Lists of full tiles of 4- and 8-byte elements with 1.75 times (f32: twice)
+// the data that the L2 cache holds and targets that are not one contiguous run per
+// tile: every kind, or for f64 the kinds in kAlignedPatchKinds, run on patches
+// (if every problem has them), the other f64 kinds on the tiles, unless some
+// are misaligned (two or three launches: a
 // submatrix, 6001 x 4999, 2% misaligned, T beta = 0.7 150 -> 134) or, for the
-// general beta, TMA could stage less than three quarters of them.  Same box, 8192^2, BC64 -> BC128, tiles -> patches:
+// general beta, TMA could stage less than three quarters of them.  Same box,
+// 8192^2, BC64 -> BC128, tiles -> patches:
 // f64 T copy 172 -> 162, T beta = 0.5 250 -> 242, N beta = 0.5 257 -> 242, but
 // alpha = 1.5 171 -> 176 and beta = 0.7 263 (TMA) -> 271; c64 T copy 171 ->
 // 161, N beta = 0.5 265 -> 241, T beta = 0.7 246 -> 242, complex beta 293 ->
-// 277.  4096^2 f64 T copy 46.3 -> 44.5; 2048^2 (in L2) 13.4 -> 14.6.  Targets
+// 277.  4096^2 f64 T copy 46.3 -> 44.5; 3072^2 25.9 -> 27.7, 2048^2 13.4 -> 14.6.  Targets
 // of 16-row panels (one run per tile) 1900 -> 1885 with three times the list.
-// c128: copy 1321 -> 1329 (16384^2), f32: copy 88 -> 103, stay on the tiles.
+// f32 T copy 87 -> 84, T beta = 0.7 135 -> 130, N beta = 0.5 130 -> 127, 64
+// matrices of 2048 x 3072 515 -> 489, 7001 x 6003 T copy 64 -> 56, N beta = 0.5
+// 94 -> 85; but 4096^2 T copy 23.8 -> 24.6, and one 8192^2 matrix (columns 32 KB
+// apart) T 89 -> 95, and cells below three quarters of a patch whose extents
+// are no multiples of 16 (BC24 -> BC100) T copy 110 -> 127: these stay.  f32
+// copies stay where transposed patches take more than 1.25 cells on average
+// (BC48 -> BC96 copy 88 -> 101, beta = 0.5 133 -> 132; BC56 -> BC112 89 -> 107,
+// 142 -> 135), and every kind if A's blocks are the smaller ones, below 7000^2
+// (BC96 -> BC32 6144^2 beta = 0.5 74 -> 75).  c128 copy (16384^2) 1321 -> 1329 stays on the tiles.
 // COSTA_PATCH=0 turns the patches off, COSTA_PATCH=1 takes them for every
 // pair that has them (for measurements).
 // Returns the kinds that run on patches (bit per kind; 0: no patches).
 // `rest`: the tiles left in `list` are other problems' than the patches'
 // (reason 1), not the same problems' for the other kinds.
 constexpr uint32_t kAllKinds = (1u << K_NKINDS) - 1u;
-constexpr uint32_t kAlignedPatchKinds = (1u << K_COPY) | (1u << K_AXPBY2);  // f64; c64: all
+constexpr uint32_t kAlignedPatchKinds = (1u << K_COPY) | (1u << K_AXPBY2);  // f64; f32, c64: all
 constexpr int64_t kL2Bytes = int64_t(126) << 20;
+
+// Whether the larger of A's and op(B)'s (first) blocks is, along some axis,
+// no power of two times the smaller one.
+bool uneven(const ProblemHost &ph) {
+    const costa_layout_s &A = *ph.A, &B = *ph.B;
+    const bool t = ph.op != COSTA_OP_N;
+    auto odd = [](int64_t a, int64_t b) {
+        const int64_t lo = std::max<int64_t>(std::min(a, b), 1), q = std::max(a, b) / lo;
+        return lo * q != std::max(a, b) || (q & (q - 1)) != 0;
+    };
+    return odd(A.R[1] - A.R[0], t ? B.C[1] - B.C[0] : B.R[1] - B.R[0]) ||
+           odd(A.C[1] - A.C[0], t ? B.R[1] - B.R[0] : B.C[1] - B.C[0]);
+}
 
 uint32_t take_patches(const Plan &plan, std::vector<TileDesc> &list, PatchList &out, bool &rest) {
     static const int mode = [] {
@@ -424,7 +463,8 @@ uint32_t take_patches(const Plan &plan, std::vector<TileDesc> &list, PatchList &
     if (mode == 0 || list.empty()) return 0;
     const int es = plan.esize;
     const bool cplx = plan.dtype == COSTA_C64 || plan.dtype == COSTA_C128;
-    int64_t all = 0, poor = 0, mis = 0, runs = 0, boxes = 0, small = 0;
+    int64_t all = 0, poor = 0, mis = 0, runs = 0, boxes = 0, small = 0, src_mis = 0, part = 0, neat = 0,
+            coarse = 0, fine = 0, trans = 0, odd16 = 0;
     for (const ProblemHost &ph : plan.probs) all += ph.A->m * ph.A->n;
     const bool many = all >= 3000000;
     for (const TileDesc &d : list) {
@@ -439,36 +479,83 @@ uint32_t take_patches(const Plan &plan, std::vector<TileDesc> &list, PatchList &
         const bool partial = es != 4 && 4 * e < 3 * int64_t(plan.ts) * plan.ts && !run;
         if (misaligned || (!along && (partial || sm))) poor += e;
         if (misaligned) mis += e;
+        else if (!(d.flags & TF_FAST)) src_mis += e;
         if (sm) small += e;
+        if ((d.nx % 16 != 0 || d.ny % 16 != 0) && 4 * e < 3 * 32 * 32) part += e;  // of a 4-byte patch
+        if ((d.flags & TF_FAST) && d.nx >= 8 && d.ny >= 8 && (d.nx & (d.nx - 1)) == 0 && (d.ny & (d.ny - 1)) == 0)
+            neat += e;
+        const ProblemHost &ph = plan.probs[d.prob];
+        const int64_t na = int64_t(ph.A->nbr) * ph.A->nbc, nb = int64_t(ph.B->nbr) * ph.B->nbc;
+        if (2 * nb <= na) coarse += e;
+        if (2 * na <= nb) fine += e;
+        if (tr) trans += e;
+        if (tr && (d.flags & TF_FAST) && d.nx >= 16 && d.ny >= 16 && uneven(ph)) odd16 += e;
         if (run) runs += e;
         const int nr = tr ? d.nx : d.ny, len = tr ? d.ny : d.nx;
         if (!misaligned && (nr == 16 || nr == 32) && len * es % 128 == 0) boxes += e;  // could be staged by TMA
     }
     const size_t n = plan.probs.size();
+    const bool beyond = 8 * all * es > (es == 8 ? 7 : 8) * kL2Bytes;  // B and A: 1.75 or 2 times the L2
     if (2 * poor >= all || (es == 8 && 20 * mis >= all) || mode == 1) {
         std::vector<char> taken(n, 0);
         bool any = false;
         for (size_t k = 0; k < n; ++k)
             any |= (taken[k] = append_patches(plan.probs[k], static_cast<int>(k), all, out)) != 0;
         if (!any) return 0;
+        uint32_t stay = 0;
+        if (es == 8 && mis == 0 && all >= 2400000 && mode != 1 && std::find(taken.begin(), taken.end(), 0) == taken.end()) {
+            const bool lines_shared = 2 * coarse >= all && 2 * trans < all;
+            if (!cplx && 4 * neat >= 3 * all) {
+                if (all < (lines_shared ? 8000000 : 20000000)) stay |= 1u << K_AXPBY2;
+                if (all < (lines_shared ? 8000000 : 50000000)) stay |= 1u << K_AXPBY;
+                if (all >= 10000000 && ((2 * fine >= all && all < 50000000) ||
+                                       (2 * coarse >= all && !lines_shared && all < 20000000)))
+                    stay |= 1u << K_SCALE;
+            }
+            if (2 * small < all && !beyond) stay |= 1u << K_COPY;
+        }
+        if (es == 4 && mis == 0 && 4 * odd16 >= 3 * all && all >= 2400000 && mode != 1 &&
+            std::find(taken.begin(), taken.end(), 0) == taken.end())
+            stay = 2 * coarse >= all ? kAllKinds : (1u << K_COPY) | (1u << K_SCALE);
+        if (stay == kAllKinds) {
+            out.patches.clear();
+            out.cells.clear();
+            return 0;
+        }
+        if (stay) {
+            rest = false;
+            return kAllKinds & ~stay;
+        }
         size_t w = 0;
         for (const TileDesc &d : list)
             if (!taken[d.prob]) list[w++] = d;
         list.resize(w);
         return kAllKinds;
     }
-    if (es != 8 || 2 * all * es <= kL2Bytes || 2 * runs >= all || 4 * small >= all || tma_mode() == 1) return 0;
+    if (es == 16 || !beyond || 2 * runs >= all || 2 * small >= all ||
+        2 * src_mis >= all || (es == 4 && 2 * part >= all) || tma_mode() == 1)
+        return 0;
+    if (es == 4)  // transposed sources whose columns lie a multiple of 32 KB apart
+        for (const ProblemHost &ph : plan.probs)
+            if (!ph.B->blocks.empty() && static_cast<int64_t>(ph.B->blocks[0].ld) * es % 32768 == 0) return 0;
     for (size_t k = 0; k < n; ++k)
         if (!append_patches(plan.probs[k], static_cast<int>(k), all, out)) {
             out.patches.clear();
             out.cells.clear();
             return 0;
         }
-    if (cplx || mis > 0) {
+    const bool cut = es == 4 && 4 * trans >= 3 * all && 4 * out.cells.size() > 5 * out.patches.size();
+    if (cut && 2 * coarse >= all && all < 50000000) {
+        out.patches.clear();
+        out.cells.clear();
+        return 0;
+    }
+    if (!cut && (es == 4 || cplx || mis > 0)) {
         list.clear();
         return kAllKinds;
     }
     rest = false;
+    if (cut) return kAllKinds & ~((1u << K_COPY) | (1u << K_SCALE));
     return kAlignedPatchKinds | (4 * boxes < 3 * all ? 1u << K_AXPBY : 0u);
 }
 
@@ -545,7 +632,7 @@ costa_status build_plan(int n, const costa_layout *As, const costa_layout *Bs, c
     // The aligned tiles also as x-halves (see use_halves), for the kinds
     // that run on them (see launch_list in transform_impl).
     std::vector<char> halve(static_cast<size_t>(n), 0);
-    for (int k = 0; k < n; ++k) halve[k] = rest && use_halves(plan->probs[k], es);
+    for (int k = 0; k < n; ++k) halve[k] = (rest || es == 4 || !((patch_kinds >> K_AXPBY2) & 1u)) && use_halves(plan->probs[k], es);
     std::vector<TileDesc> halves = split_x_halves(split.big, ts / 2, es, halve);
     const bool had_halves = !halves.empty();
     split.big = cut_few(std::move(split.big), es);
