@@ -50,6 +50,13 @@ from workloads.materialize import DeviceMatrix, HostMatrix  # noqa: E402
 L2_BYTES = 129 * 1024 * 1024
 KERNEL_SOURCES = ["paper_2106_06601_gb300/csrc/remap_impl.cuh",
                   "paper_2106_06601_gb300/csrc/fxdot.h",  # fixed-point sums of the complex kinds
+                  "paper_2106_06601_gb300/csrc/remap_patch.cuh",
+                  "paper_2106_06601_gb300/csrc/rnmul.h",  # products on the integer pipes
+                  "paper_2106_06601_gb300/csrc/patches.cpp",  # patches and their order
+                  "paper_2106_06601_gb300/csrc/patch_f64.cu",
+                  "paper_2106_06601_gb300/csrc/patch_f32.cu",
+                  "paper_2106_06601_gb300/csrc/patch_c64.cu",
+                  "paper_2106_06601_gb300/csrc/patch_c128.cu",
                   "paper_2106_06601_gb300/csrc/remap_f64.cu",
                   "paper_2106_06601_gb300/csrc/remap_f32.cu",
                   "paper_2106_06601_gb300/csrc/remap_c64.cu",
