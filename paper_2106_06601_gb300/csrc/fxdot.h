@@ -15,7 +15,8 @@
 //      U = 2^-7 ulp(M) or finer (M the largest product): dropping and
 //      alignment together truncate less than one U per product;
 //   3. the integer sum is rounded once to double, to nearest even, by the
-//      hardware's conversion, and the exponent added to its exponent field.
+//      hardware's conversion or on the integer pipes (the same bits), and the
+//      exponent added to its exponent field.
 // The result is within 0.5 ulp(x) + n U of the exact sum x of the n exact
 // products: n U <= 2^-5 ulp(M), so at most 0.5 ulp(x) + 0.032 ulp(M).  All
 // intermediate magnitudes stay in the normal range: a product lies in
@@ -82,6 +83,14 @@ COSTA_FX_HD uint64_t shr_clamp(uint64_t v, uint32_t n) {
 #endif
 }
 
+COSTA_FX_HD uint32_t leading_zeros(uint64_t v) {
+#ifdef __CUDA_ARCH__
+    return static_cast<uint32_t>(__clzll(static_cast<long long>(v)));
+#else
+    return static_cast<uint32_t>(__builtin_clzll(v));
+#endif
+}
+
 // The integer rounded to the nearest double, ties to even.
 COSTA_FX_HD double round_to_double(int64_t v) {
 #ifdef __CUDA_ARCH__
@@ -89,6 +98,19 @@ COSTA_FX_HD double round_to_double(int64_t v) {
 #else
     return static_cast<double>(v);  // the default rounding mode is to nearest even
 #endif
+}
+
+// The same, |v| < 2^63, without the conversion, for the complex-alpha kind: its
+// other component is formed on the FP64 pipe, and the conversions' rate is as
+// low.  GB300, c128 BC64 -> BC128 T, complex alpha, us per call, conversion ->
+// this: 2048^2 56.2 -> 49.6, 4096^2 173.0 -> 147.9; but with a complex beta, one
+// component of two so, 233 -> 256 (the ALU pipe bounds it).
+COSTA_FX_HD uint64_t round_to_double_bits_alu(int64_t v) {
+    const uint64_t neg = static_cast<uint64_t>(v >> 63), mag = (static_cast<uint64_t>(v) ^ neg) - neg;
+    const uint32_t lz = leading_zeros(mag | 1u);  // >= 1
+    const uint64_t m = mag << (lz - 1u);        // leading bit at 62
+    const uint64_t q = (m + 0x1FFu + ((m >> 10) & 1u)) >> 10;  // 53 bits, ties to even; a carry moves on to the exponent
+    return (neg << 63) + ((static_cast<uint64_t>(1085u - lz) << 52) + q);
 }
 
 // An operand: its 53-bit significand as 31 top bits (h) and 22 low bits at the
@@ -142,8 +164,8 @@ COSTA_FX_HD Term mul(const Op &x, const Op &y, uint32_t neg) {
 }
 
 // The sum of n <= 4 terms, rounded once to double (to nearest, ties to even).
-// A zero sum gives +0.
-template <int N>
+// A zero sum gives +0.  ALU: rounded without the hardware's conversion.
+template <bool ALU = false, int N>
 COSTA_FX_HD double sum(const Term (&t)[N]) {
     int32_t emax = t[0].e;
 #pragma unroll
@@ -161,7 +183,8 @@ COSTA_FX_HD double sum(const Term (&t)[N]) {
     if (acc == 0) return 0.0;
     // acc's unit is 2^(emax - 2105): a significand product has unit
     // 2^(emax - 2150), and acc's is 2^45 of it
-    const uint64_t r = bits_of(round_to_double(static_cast<int64_t>(acc)));
+    const uint64_t r = ALU ? round_to_double_bits_alu(static_cast<int64_t>(acc))
+                           : bits_of(round_to_double(static_cast<int64_t>(acc)));
     return from_bits(r + (static_cast<uint64_t>(static_cast<int64_t>(emax - 2105)) << 52));
 }
 

@@ -97,7 +97,8 @@ template <> struct ET<double2> { enum { VEC = 1, CPLX = 1 }; typedef double R; }
 //    with Kahan's algorithm alone): T and N 1458 -> 2133 with 2 to 4
 //    blocks; with half of the components summed in fixed point on the integer
 //    pipes, unrolled, 2557 at 2 blocks, 2660 at 3 (a third or a quarter of
-//    them: 2553, 2569); in the rolled loop, 3 blocks, 3259.
+//    them: 2553, 2569); in the rolled loop, 3 blocks, 3259; with their
+//    imaginary components' sums rounded on the integer pipes too, 3630.
 //  - c64 complex scalars, against 3 blocks with 2 buffers: complex beta
 //    T 4484 -> 5482, N 4495 -> 5495 with 4 blocks and no look-ahead;
 //    complex alpha T 5551 -> 5955 with two tiles ahead; the real general
@@ -502,7 +503,7 @@ __device__ __forceinline__ double2 mid_cscale(const double2 &b, const Sc &s) {
     const fx::Term im[2] = {fx::mul(far, fby, 0u), fx::mul(fai, fbx, 0u)};  // ar by + ai bx
     double2 o;
     o.x = kahan2(s.ar, b.x, s.ai, b.y, true);  // ar bx - ai by
-    o.y = fx::sum(im);
+    o.y = fx::sum<true>(im);
     return o;
 }
 
