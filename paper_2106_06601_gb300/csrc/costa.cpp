@@ -1236,6 +1236,7 @@ Scalars make_scalars(int dt, const void *alpha, const void *beta, int index) {
     if (s.beta[0] == 0.0 && s.beta[1] == 0.0) s.flags |= SF_BETA0;
     if (s.alpha[0] == 1.0 && s.alpha[1] == 0.0) s.flags |= SF_ALPHA1;
     if (s.alpha[1] != 0.0 || s.beta[1] != 0.0) s.flags |= SF_CPLX;
+    if (dt == COSTA_C128 && s.alpha[1] == 0.0) s.flags |= SF_AREAL;
     int e = 0;
     const double fr = std::frexp(std::fabs(s.beta[0]), &e);
     if (s.beta[1] == 0.0 && fr == 0.5 && e - 1 >= -1000 && e - 1 <= 1000) {

@@ -127,7 +127,7 @@ struct Scalars {
     int32_t flags;
     int32_t beta_exp;  // k with |beta| = 2^k when SF_BPOW2 is set
 };
-enum : int32_t { SF_BETA0 = 1, SF_ALPHA1 = 2, SF_CPLX = 4, SF_BPOW2 = 8 };
+enum : int32_t { SF_BETA0 = 1, SF_ALPHA1 = 2, SF_CPLX = 4, SF_BPOW2 = 8, SF_AREAL = 16 };
 
 // Combine kinds: each kernel is compiled for one, so every path keeps only
 // the registers it needs.
@@ -136,19 +136,22 @@ enum : int32_t { SF_BETA0 = 1, SF_ALPHA1 = 2, SF_CPLX = 4, SF_BPOW2 = 8 };
 //   K_AXPBY real alpha, beta != 0      out = fma(alpha, op(b), beta * a)
 //   K_CPLX  complex beta (or complex alpha with beta != 0): each component
 //           a compensated sum of its four products (Dot2)
+//   K_CPLXR as K_CPLX for double complex data and a real alpha (SF_AREAL): the
+//            same bits without the two products that are zero
 //   K_AXPBY2 as K_AXPBY with beta = +-2^k: beta * a is formed exactly on the
 //            integer pipes (exponent add), saving one multiply on the scarce
 //            FP64 pipe; same bits as K_AXPBY
 //   K_CSCALE complex alpha, beta = 0   out = alpha * op(b) by Dot2 (double
 //            data in the middle range: Kahan's 2 x 2 determinant algorithm);
 //            A is not read (BLAS convention), so NaN in A does not propagate
-enum : int { K_COPY = 0, K_SCALE = 1, K_AXPBY = 2, K_CPLX = 3, K_AXPBY2 = 4, K_CSCALE = 5, K_NKINDS = 6 };
+enum : int { K_COPY = 0, K_SCALE = 1, K_AXPBY = 2, K_CPLX = 3, K_AXPBY2 = 4, K_CSCALE = 5, K_CPLXR = 6, K_NKINDS = 7 };
 
 // The kinds whose output depends on A's old value (beta != 0).
-COSTA_HD constexpr bool kind_reads_a(int kind) { return kind == K_AXPBY || kind == K_CPLX || kind == K_AXPBY2; }
+COSTA_HD constexpr bool kind_cplx(int kind) { return kind == K_CPLX || kind == K_CPLXR; }
+COSTA_HD constexpr bool kind_reads_a(int kind) { return kind == K_AXPBY || kind_cplx(kind) || kind == K_AXPBY2; }
 
 COSTA_HD inline int kind_of(int32_t flags) {
-    if (flags & SF_CPLX) return (flags & SF_BETA0) ? K_CSCALE : K_CPLX;
+    if (flags & SF_CPLX) return (flags & SF_BETA0) ? K_CSCALE : (flags & SF_AREAL) ? K_CPLXR : K_CPLX;
     if (!(flags & SF_BETA0)) return (flags & SF_BPOW2) ? K_AXPBY2 : K_AXPBY;
     if (!(flags & SF_ALPHA1)) return K_SCALE;
     return K_COPY;

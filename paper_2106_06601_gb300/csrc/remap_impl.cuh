@@ -122,7 +122,9 @@ template <> struct ET<double2> { enum { VEC = 1, CPLX = 1 }; typedef double R; }
 //    at a time, 1186 with 2, 1194 with 4, instruction fetch the limit;
 //    rolled: 2286 with 1, 2340 with 2 at 136 registers and 3 blocks, 2115
 //    with 4).  With the sums' shorter form (fxdot.h), 4096^2: 2 blocks 292
-//    us, 3 blocks 234, 4 blocks 238 (spills); 1, 2, 3 passes 264, 234, 252.
+//    us, 3 blocks 234, 4 blocks 238 (spills); 1, 2, 3 passes 264, 234, 252;
+//    with a real alpha (K_CPLXR) 207 (one kernel for both: 217, and 240 with
+//    a complex alpha).
 // Each entry is overridable at build time for tuning (COSTA_WARPS_4/8,
 // COSTA_MINB_* and COSTA_NBUF_*).
 #ifndef COSTA_WARPS_4
@@ -227,12 +229,12 @@ constexpr Shape launch_shape(int es, bool cplx, int kind, bool mis) {
     const bool reads_a = kind_reads_a(kind);
     if (es == 4) return reads_a ? Shape{COSTA_MINB_4A, COSTA_NBUF_4A} : Shape{COSTA_MINB_4, COSTA_NBUF_4};
     if (es == 16) {
-        if (kind == K_CPLX) return {COSTA_MINB_16C, COSTA_NBUF_16A};
+        if (kind_cplx(kind)) return {COSTA_MINB_16C, COSTA_NBUF_16A};
         if (reads_a) return {COSTA_MINB_16A, COSTA_NBUF_16A};
         if (kind == K_CSCALE) return {COSTA_MINB_16CS, COSTA_NBUF_16CS};
         return kind == K_SCALE ? Shape{COSTA_MINB_16S, COSTA_NBUF_16S} : Shape{COSTA_MINB_16, COSTA_NBUF_16};
     }
-    if (kind == K_CPLX) return {COSTA_MINB_8C, COSTA_NBUF_8C};
+    if (kind_cplx(kind)) return {COSTA_MINB_8C, COSTA_NBUF_8C};
     if (kind == K_CSCALE) return {COSTA_MINB_8CS, COSTA_NBUF_8CS};
     if (kind == K_AXPBY) return {COSTA_MINB_8H, COSTA_NBUF_8H};
     if (mis) {
@@ -267,7 +269,7 @@ template <typename T> struct Cfg {
 };
 
 template <typename T, int KIND, bool MIS = false> struct KCfg {
-    static constexpr bool HEAVY = KIND == K_AXPBY || KIND == K_CPLX || KIND == K_CSCALE;
+    static constexpr bool HEAVY = KIND == K_AXPBY || kind_cplx(KIND) || KIND == K_CSCALE;
     static constexpr bool READS_A = kind_reads_a(KIND);
     static constexpr int WARPS = Cfg<T>::WARPS;
     static constexpr Shape SHAPE = launch_shape(static_cast<int>(sizeof(T)), ET<T>::CPLX != 0, KIND, MIS);
@@ -477,16 +479,25 @@ template <typename C> __device__ __forceinline__ bool cplx_mid(const C &, const 
 // (fxdot.h): within 0.5 ulp of the component plus 2^-5 ulp of its largest
 // product, with no FP64 operation.  Dot2 takes 24 FP64 operations per
 // component, and the FP64 pipe is narrow on GB300.  Every operand must be in
-// the middle range (cplx_mid).
+// the middle range (cplx_mid).  REAL (K_CPLXR): alpha's imaginary part is zero,
+// and so are its products, which leave a sum's bits as they are.
+template <bool REAL>
 __device__ __forceinline__ double2 fx_cplx(const double2 &b, const double2 &a, const Sc &s) {
     const fx::Op fbx = fx::unpack(b.x), fby = fx::unpack(b.y), fax = fx::unpack(a.x), fay = fx::unpack(a.y);
     const fx::Op far = fx::unpack(s.ar), fai = fx::unpack(s.ai), fbr = fx::unpack(s.br), fbi = fx::unpack(s.bi);
+    double2 o;
+    if constexpr (REAL) {
+        const fx::Term re[3] = {fx::mul(far, fbx, 0u), fx::mul(fbr, fax, 0u), fx::mul(fbi, fay, 1u)};
+        const fx::Term im[3] = {fx::mul(far, fby, 0u), fx::mul(fbr, fay, 0u), fx::mul(fbi, fax, 0u)};
+        o.x = fx::sum(re);
+        o.y = fx::sum(im);
+        return o;
+    }
     // ar bx - ai by + br ax - bi ay;  ar by + ai bx + br ay + bi ax
     const fx::Term re[4] = {fx::mul(far, fbx, 0u), fx::mul(fai, fby, 1u), fx::mul(fbr, fax, 0u),
                             fx::mul(fbi, fay, 1u)};
     const fx::Term im[4] = {fx::mul(far, fby, 0u), fx::mul(fai, fbx, 0u), fx::mul(fbr, fay, 0u),
                             fx::mul(fbi, fax, 0u)};
-    double2 o;
     o.x = fx::sum(re);
     o.y = fx::sum(im);
     return o;
@@ -511,7 +522,7 @@ template <int KIND, typename C, typename R>
 __device__ __forceinline__ C combine_c(C b, C a, const Sc &s) {
     b.y = flip_sign(b.y, s.conj_mask);
     C o;
-    if (KIND != K_CPLX && KIND != K_CSCALE) {
+    if (!kind_cplx(KIND) && KIND != K_CSCALE) {
         o.x = comb_real<KIND, R>(b.x, a.x, s);
         o.y = comb_real<KIND, R>(b.y, a.y, s);
         return o;
@@ -521,16 +532,16 @@ __device__ __forceinline__ C combine_c(C b, C a, const Sc &s) {
         // Dot2 below
         if (s.alpha_mid && mid_range(b.x) && mid_range(b.y)) return mid_cscale(b, s);
     }
-    if constexpr (KIND == K_CPLX && sizeof(R) == 8) {
+    if constexpr (kind_cplx(KIND) && sizeof(R) == 8) {
         // four-term components: in fixed point on the integer pipes when
         // every operand is in the middle range (fx_cplx)
-        if (cplx_mid(b, a, s)) return fx_cplx(b, a, s);
+        if (cplx_mid(b, a, s)) return fx_cplx<KIND == K_CPLXR>(b, a, s);
     }
     const R ar = R(s.ar), ai = R(s.ai);
     Dot2<R> re(ar, b.x), im(ar, b.y);
     re.add(-ai, b.y);
     im.add(ai, b.x);
-    if (KIND == K_CPLX) {
+    if (kind_cplx(KIND)) {
         const R br = R(s.br), bi = R(s.bi);
         re.add(br, a.x);
         re.add(-bi, a.y);
@@ -733,7 +744,7 @@ __device__ __forceinline__ unsigned char *slot_any(unsigned char *buf, int r, in
 // few passes ahead (stage_drain); for the other kinds that read A the
 // caller loads the tile's A chunks into registers first (load_a).
 template <typename T, int KIND> __host__ __device__ constexpr bool drain_loads_a() {
-    return KIND == K_CPLX && sizeof(T) == 16;
+    return kind_cplx(KIND) && sizeof(T) == 16;
 }
 
 // Write a staged fast tile to A, combining with A when the kind reads it.
@@ -746,7 +757,7 @@ __device__ __forceinline__ void stage_drain(const Geom<T> &g, const Sc &s, unsig
     if (m.c >= chunks) return;
     const int x0 = m.c * C::VEC;
     const int npass = (g.ny + m.rpp - 1) / m.rpp;
-    if constexpr ((KIND == K_CPLX || KIND == K_CSCALE) && sizeof(T) == 16) {
+    if constexpr ((kind_cplx(KIND) || KIND == K_CSCALE) && sizeof(T) == 16) {
         // double complex with complex scalars: G passes at a time in
         // straight-line code, so that their evaluations overlap.  Four-term
         // components (complex beta) are all summed in fixed point on the
@@ -765,7 +776,7 @@ __device__ __forceinline__ void stage_drain(const Geom<T> &g, const Sc &s, unsig
             for (int j = 0; j < G; ++j) {
                 const int y = (q0 + j) * m.rpp + m.r0;
                 dst[j] = T{0.0, 0.0};
-                if (KIND == K_CPLX && q0 + j < npass && y < g.ny)
+                if (kind_cplx(KIND) && q0 + j < npass && y < g.ny)
                     dst[j] = load_rw(g.dst + static_cast<int64_t>(y) * g.dld + x0).e[0];
             }
         };
@@ -790,15 +801,15 @@ __device__ __forceinline__ void stage_drain(const Geom<T> &g, const Sc &s, unsig
                               : T{0.0, 0.0};
                 bb[j].y = flip_sign(bb[j].y, s.conj_mask);
             }
-            bool mid = KIND == K_CPLX || s.alpha_mid;
+            bool mid = kind_cplx(KIND) || s.alpha_mid;
 #pragma unroll
             for (int j = 0; j < G; ++j)
-                mid = mid && (KIND == K_CPLX ? cplx_mid(bb[j], aa[j], s) : mid_range(bb[j].x) && mid_range(bb[j].y));
+                mid = mid && (kind_cplx(KIND) ? cplx_mid(bb[j], aa[j], s) : mid_range(bb[j].x) && mid_range(bb[j].y));
             T o[G];
             if (mid) {
 #pragma unroll
                 for (int j = 0; j < G; ++j) {
-                    o[j] = KIND == K_CPLX ? fx_cplx(bb[j], aa[j], s) : mid_cscale(bb[j], s);
+                    o[j] = kind_cplx(KIND) ? fx_cplx<KIND == K_CPLXR>(bb[j], aa[j], s) : mid_cscale(bb[j], s);
                 }
             } else {
 #pragma unroll
@@ -1869,6 +1880,9 @@ cudaError_t launch_remap_t(const RemapLaunch &a, int kind, cudaStream_t st) {
     case K_AXPBY2: return launch_t<T, K_AXPBY2>(a, st);
     case K_CPLX:
         if constexpr (ET<T>::CPLX) return launch_t<T, K_CPLX>(a, st);
+        return cudaErrorInvalidValue;
+    case K_CPLXR:
+        if constexpr (sizeof(T) == 16) return launch_t<T, K_CPLXR>(a, st);
         return cudaErrorInvalidValue;
     case K_CSCALE:
         if constexpr (ET<T>::CPLX) return launch_t<T, K_CSCALE>(a, st);

@@ -76,7 +76,7 @@ namespace remap {
 constexpr int patch_blocks(int es, bool cplx, int kind) {
     const bool reads_a = kind_reads_a(kind);
     if (es == 4) return reads_a ? COSTA_PB_4A : COSTA_PB_4;
-    if (es == 16) return kind == K_CPLX || kind == K_CSCALE ? COSTA_PB_16C : COSTA_PB_16;
+    if (es == 16) return kind_cplx(kind) || kind == K_CSCALE ? COSTA_PB_16C : COSTA_PB_16;
     return reads_a ? COSTA_PB_8A : kind == K_SCALE && !cplx ? COSTA_PB_8S : COSTA_PB_8;
 }
 
@@ -101,7 +101,7 @@ template <typename T, int KIND> struct PCfg {
     // complex scalars on double complex data: two passes together, rolled (the
     // fixed-point sums are long; BC50 -> BC75, 4096^2, complex beta, one, two,
     // four passes: 306, 276, 322 us)
-    static constexpr bool ROLLED = ES == 16 && (KIND == K_CPLX || KIND == K_CSCALE);
+    static constexpr bool ROLLED = ES == 16 && (kind_cplx(KIND) || KIND == K_CSCALE);
     // passes whose elements of A are loaded together: the whole patch in two
     // groups, a quarter for 8-byte elements (registers)
     static constexpr int G = ROLLED ? COSTA_PGR : ES == 4 ? 16 : ES == 8 ? 8 : 4;
@@ -459,6 +459,9 @@ cudaError_t launch_patch_t(const PatchLaunch &a, int kind, cudaStream_t st) {
     case K_AXPBY2: return launch_patch<T, K_AXPBY2>(a, st);
     case K_CPLX:
         if constexpr (ET<T>::CPLX) return launch_patch<T, K_CPLX>(a, st);
+        return cudaErrorInvalidValue;
+    case K_CPLXR:
+        if constexpr (sizeof(T) == 16) return launch_patch<T, K_CPLXR>(a, st);
         return cudaErrorInvalidValue;
     case K_CSCALE:
         if constexpr (ET<T>::CPLX) return launch_patch<T, K_CSCALE>(a, st);

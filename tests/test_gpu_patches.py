@@ -13,7 +13,7 @@ pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
 KINDS = {"copy": (1.0, 0.0), "scale": (-0.7, 0.0), "axpby": (-0.3, 0.7), "axpby2": (2.0, -0.5)}
-CPLX_KINDS = {"cplx": (complex(1.0, 0.5), complex(0.5, -0.25)), "cscale": (complex(0.3, -0.4), 0.0)}
+CPLX_KINDS = {"cplx": (complex(1.0, 0.5), complex(0.5, -0.25)), "cplxr": (-1.5, complex(0.3, 0.7)), "cscale": (complex(0.3, -0.4), 0.0)}
 #         m, n      source      target      grids   pads
 SHAPES = (((1, 97), (5, 7), (3, 11), (1, 2), (0, 1)), ((97, 1), (5, 7), (3, 11), (2, 1), (1, 0)),
           ((33, 31), (50, 50), (75, 75), (1, 1), (1, 1)), ((65, 130), (1, 2), (3, 1), (2, 2), (0, 0)),
