@@ -465,7 +465,13 @@ uint32_t take_patches(const Plan &plan, std::vector<TileDesc> &list, PatchList &
     const bool cplx = plan.dtype == COSTA_C64 || plan.dtype == COSTA_C128;
     int64_t all = 0, poor = 0, mis = 0, runs = 0, boxes = 0, small = 0, src_mis = 0, part = 0, neat = 0,
             coarse = 0, fine = 0, trans = 0, odd16 = 0;
-    for (const ProblemHost &ph : plan.probs) all += ph.A->m * ph.A->n;
+    std::vector<char> ratio;  // per problem: 1 B's blocks the larger ones, 2 A's, 4 uneven
+    ratio.reserve(plan.probs.size());
+    for (const ProblemHost &ph : plan.probs) {
+        all += ph.A->m * ph.A->n;
+        const int64_t na = int64_t(ph.A->nbr) * ph.A->nbc, nb = int64_t(ph.B->nbr) * ph.B->nbc;
+        ratio.push_back(static_cast<char>((2 * nb <= na ? 1 : 0) | (2 * na <= nb ? 2 : 0) | (uneven(ph) ? 4 : 0)));
+    }
     const bool many = all >= 3000000;
     for (const TileDesc &d : list) {
         const int64_t e = static_cast<int64_t>(d.nx) * d.ny;
@@ -484,12 +490,11 @@ uint32_t take_patches(const Plan &plan, std::vector<TileDesc> &list, PatchList &
         if ((d.nx % 16 != 0 || d.ny % 16 != 0) && 4 * e < 3 * 32 * 32) part += e;  // of a 4-byte patch
         if ((d.flags & TF_FAST) && d.nx >= 8 && d.ny >= 8 && (d.nx & (d.nx - 1)) == 0 && (d.ny & (d.ny - 1)) == 0)
             neat += e;
-        const ProblemHost &ph = plan.probs[d.prob];
-        const int64_t na = int64_t(ph.A->nbr) * ph.A->nbc, nb = int64_t(ph.B->nbr) * ph.B->nbc;
-        if (2 * nb <= na) coarse += e;
-        if (2 * na <= nb) fine += e;
+        const int r = ratio[d.prob];
+        if (r & 1) coarse += e;
+        if (r & 2) fine += e;
         if (tr) trans += e;
-        if (tr && (d.flags & TF_FAST) && d.nx >= 16 && d.ny >= 16 && uneven(ph)) odd16 += e;
+        if ((r & 4) && tr && (d.flags & TF_FAST) && d.nx >= 16 && d.ny >= 16) odd16 += e;
         if (run) runs += e;
         const int nr = tr ? d.nx : d.ny, len = tr ? d.ny : d.nx;
         if (!misaligned && (nr == 16 || nr == 32) && len * es % 128 == 0) boxes += e;  // could be staged by TMA

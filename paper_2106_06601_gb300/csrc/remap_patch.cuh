@@ -1,6 +1,7 @@
 // The patch kernel of the reshuffle (combine kinds, staging and launch idiom
 // as in remap_impl.cuh): it moves pairs whose grid-overlay cells are mostly
-// small or whose runs start off 16-byte boundaries.
+// small or whose runs start off 16-byte boundaries, and large lists of 4- and
+// 8-byte elements (take_patches in costa.cpp has the rule).
 //
 // What bounds the tile kernel there: a tile lies in one overlay cell, so
 // small or odd cells leave lanes idle, bytes out of flight and a descriptor
@@ -13,7 +14,7 @@
 //      own alignment, so any phase is the same case), lanes along the
 //      source's contiguous axis, one run per step of the other axis; a lane
 //      reads its cell's address when a segment starts and adds the stride
-//      after that;
+//      after that (4-byte runs of whole aligned 16-byte chunks: by chunks);
 //   3. the warp writes A one run per step, one element per lane, reading the
 //      staged rows across (transposed) or along; an odd row pitch keeps both
 //      free of bank conflicts and the addresses free of swizzles.
@@ -163,8 +164,8 @@ __device__ __forceinline__ int chunk_slot(int r, int c) { return r * 128 + ((c ^
 // Copies a patch's source into `buf`, one run of the source per row.  4-byte
 // patches more than 16 elements wide whose source runs are whole aligned
 // 16-byte chunks (TF_FAST) copy those: they bypass the L1 and take a quarter of the instructions.  GB300,
-// 8192^2 f32 T, us per call, elements -> chunks: copy BC8 101 -> 84, A's ld odd
-// 109 -> 90; beta = 0.5 BC8 138 -> 130, A's ld odd 149 -> 134.
+// 8192^2 f32 T, us per call, elements -> chunks: copy BC8 101 -> 83, A's ld odd
+// 108 -> 90; beta = 0.5 BC8 138 -> 126, A's ld odd 149 -> 134.
 template <typename T, int KIND>
 __device__ __forceinline__ void patch_stage(const PatchDesc &d, const uint4 *cells, unsigned char *buf, int lane) {
     using P = PCfg<T, KIND>;
