@@ -463,8 +463,7 @@ uint32_t take_patches(const Plan &plan, std::vector<TileDesc> &list, PatchList &
     if (mode == 0 || list.empty()) return 0;
     const int es = plan.esize;
     const bool cplx = plan.dtype == COSTA_C64 || plan.dtype == COSTA_C128;
-    int64_t all = 0, poor = 0, mis = 0, runs = 0, boxes = 0, small = 0, src_mis = 0, part = 0, neat = 0,
-            coarse = 0, fine = 0, trans = 0, odd16 = 0;
+    int64_t all = 0;
     std::vector<char> ratio;  // per problem: 1 B's blocks the larger ones, 2 A's, 4 uneven
     ratio.reserve(plan.probs.size());
     for (const ProblemHost &ph : plan.probs) {
@@ -473,7 +472,11 @@ uint32_t take_patches(const Plan &plan, std::vector<TileDesc> &list, PatchList &
         ratio.push_back(static_cast<char>((2 * nb <= na ? 1 : 0) | (2 * na <= nb ? 2 : 0) | (uneven(ph) ? 4 : 0)));
     }
     const bool many = all >= 3000000;
-    for (const TileDesc &d : list) {
+    struct Sums {  // elements by what their tiles are
+        int64_t poor = 0, mis = 0, runs = 0, boxes = 0, small = 0, src_mis = 0, part = 0, neat = 0, coarse = 0, fine = 0,
+                trans = 0, odd16 = 0;
+    };
+    auto count = [&](const TileDesc &d, Sums &c) {
         const int64_t e = static_cast<int64_t>(d.nx) * d.ny;
         const bool misaligned = es == 4 ? !aligned16(d.dst, static_cast<int64_t>(d.dld) * es) || d.nx % 4 != 0
                                         : !(d.flags & TF_FAST);
@@ -483,21 +486,37 @@ uint32_t take_patches(const Plan &plan, std::vector<TileDesc> &list, PatchList &
         // in large lists, 4- and 8-byte tiles along A's runs are poor below 16 x 16 only
         const bool along = many && !tr && es < 16 && d.nx >= 16 && d.ny >= 16;
         const bool partial = es != 4 && 4 * e < 3 * int64_t(plan.ts) * plan.ts && !run;
-        if (misaligned || (!along && (partial || sm))) poor += e;
-        if (misaligned) mis += e;
-        else if (!(d.flags & TF_FAST)) src_mis += e;
-        if (sm) small += e;
-        if ((d.nx % 16 != 0 || d.ny % 16 != 0) && 4 * e < 3 * 32 * 32) part += e;  // of a 4-byte patch
+        if (misaligned || (!along && (partial || sm))) c.poor += e;
+        if (misaligned) c.mis += e;
+        else if (!(d.flags & TF_FAST)) c.src_mis += e;
+        if (sm) c.small += e;
+        if ((d.nx % 16 != 0 || d.ny % 16 != 0) && 4 * e < 3 * 32 * 32) c.part += e;  // of a 4-byte patch
         if ((d.flags & TF_FAST) && d.nx >= 8 && d.ny >= 8 && (d.nx & (d.nx - 1)) == 0 && (d.ny & (d.ny - 1)) == 0)
-            neat += e;
+            c.neat += e;
         const int r = ratio[d.prob];
-        if (r & 1) coarse += e;
-        if (r & 2) fine += e;
-        if (tr) trans += e;
-        if ((r & 4) && tr && (d.flags & TF_FAST) && d.nx >= 16 && d.ny >= 16) odd16 += e;
-        if (run) runs += e;
+        if (r & 1) c.coarse += e;
+        if (r & 2) c.fine += e;
+        if (tr) c.trans += e;
+        if ((r & 4) && tr && (d.flags & TF_FAST) && d.nx >= 16 && d.ny >= 16) c.odd16 += e;
+        if (run) c.runs += e;
         const int nr = tr ? d.nx : d.ny, len = tr ? d.ny : d.nx;
-        if (!misaligned && (nr == 16 || nr == 32) && len * es % 128 == 0) boxes += e;  // could be staged by TMA
+        if (!misaligned && (nr == 16 || nr == 32) && len * es % 128 == 0) c.boxes += e;  // could be staged by TMA
+    };
+    constexpr size_t kChunk = 1 << 16;
+    std::vector<Sums> part_sums((list.size() + kChunk - 1) / kChunk);
+    parallel_for(static_cast<int64_t>(part_sums.size()), 1, [&](int64_t k0, int64_t k1) {
+        for (int64_t k = k0; k < k1; ++k) {
+            Sums c;
+            const size_t end = std::min(list.size(), static_cast<size_t>(k + 1) * kChunk);
+            for (size_t i = static_cast<size_t>(k) * kChunk; i < end; ++i) count(list[i], c);
+            part_sums[static_cast<size_t>(k)] = c;
+        }
+    });
+    int64_t poor = 0, mis = 0, runs = 0, boxes = 0, small = 0, src_mis = 0, part = 0, neat = 0, coarse = 0, fine = 0,
+            trans = 0, odd16 = 0;
+    for (const Sums &c : part_sums) {
+        poor += c.poor, mis += c.mis, runs += c.runs, boxes += c.boxes, small += c.small, src_mis += c.src_mis;
+        part += c.part, neat += c.neat, coarse += c.coarse, fine += c.fine, trans += c.trans, odd16 += c.odd16;
     }
     const size_t n = plan.probs.size();
     const bool beyond = 8 * all * es > (es == 8 ? 7 : 8) * kL2Bytes;  // B and A: 1.75 or 2 times the L2
