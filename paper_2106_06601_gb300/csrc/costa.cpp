@@ -432,8 +432,6 @@ costa_status check_access(costa_layout_s *L, int dev, const char *which) {
 // (BC48 -> BC96 copy 88 -> 101, beta = 0.5 133 -> 132; BC56 -> BC112 89 -> 107,
 // 142 -> 135), and every kind if A's blocks are the smaller ones, below 7000^2
 // (BC96 -> BC32 6144^2 beta = 0.5 74 -> 75).  c128 copy (16384^2) 1321 -> 1329 stays on the tiles.
-// COSTA_PATCH=0 turns the patches off, COSTA_PATCH=1 takes them for every
-// pair that has them (for measurements).
 // Returns the kinds that run on patches (bit per kind; 0: no patches).
 // `rest`: the tiles left in `list` are other problems' than the patches'
 // (reason 1), not the same problems' for the other kinds.
@@ -455,12 +453,8 @@ bool uneven(const ProblemHost &ph) {
 }
 
 uint32_t take_patches(const Plan &plan, std::vector<TileDesc> &list, PatchList &out, bool &rest) {
-    static const int mode = [] {
-        const char *e = std::getenv("COSTA_PATCH");
-        return e ? std::atoi(e) : -1;
-    }();
     rest = true;
-    if (mode == 0 || list.empty()) return 0;
+    if (list.empty()) return 0;
     const int es = plan.esize;
     const bool cplx = plan.dtype == COSTA_C64 || plan.dtype == COSTA_C128;
     int64_t all = 0;
@@ -520,14 +514,14 @@ uint32_t take_patches(const Plan &plan, std::vector<TileDesc> &list, PatchList &
     }
     const size_t n = plan.probs.size();
     const bool beyond = 8 * all * es > (es == 8 ? 7 : 8) * kL2Bytes;  // B and A: 1.75 or 2 times the L2
-    if (2 * poor >= all || (es == 8 && 20 * mis >= all) || mode == 1) {
+    if (2 * poor >= all || (es == 8 && 20 * mis >= all)) {
         std::vector<char> taken(n, 0);
         bool any = false;
         for (size_t k = 0; k < n; ++k)
             any |= (taken[k] = append_patches(plan.probs[k], static_cast<int>(k), all, out)) != 0;
         if (!any) return 0;
         uint32_t stay = 0;
-        if (es == 8 && mis == 0 && all >= 2400000 && mode != 1 && std::find(taken.begin(), taken.end(), 0) == taken.end()) {
+        if (es == 8 && mis == 0 && all >= 2400000 && std::find(taken.begin(), taken.end(), 0) == taken.end()) {
             const bool lines_shared = 2 * coarse >= all && 2 * trans < all;
             if (!cplx && 4 * neat >= 3 * all) {
                 if (all < (lines_shared ? 8000000 : 20000000)) stay |= 1u << K_AXPBY2;
@@ -538,7 +532,7 @@ uint32_t take_patches(const Plan &plan, std::vector<TileDesc> &list, PatchList &
             }
             if (2 * small < all && !beyond) stay |= 1u << K_COPY;
         }
-        if (es == 4 && mis == 0 && 4 * odd16 >= 3 * all && all >= 2400000 && mode != 1 &&
+        if (es == 4 && mis == 0 && 4 * odd16 >= 3 * all && all >= 2400000 &&
             std::find(taken.begin(), taken.end(), 0) == taken.end())
             stay = 2 * coarse >= all ? kAllKinds : (1u << K_COPY) | (1u << K_SCALE);
         if (stay == kAllKinds) {
