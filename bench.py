@@ -614,22 +614,23 @@ def run_e2e(args, costa, mats, step, stream, dev, world, nbytes):
 
 
 def direct_kernels(costa, mats):
-    """Which remap kernels the direct list runs: the tile kernel, and the
-    small-tile kernel when small tiles hold at least half of the elements of
-    the (batched) list, by the planner's rule (costa_debug_split)."""
+    """Which remap kernels the direct list may run: patches where the pairs
+    have them and the planner's rule for their type, size and scalars takes
+    them (costa_debug_patches), else the tile kernel, and the small-tile kernel
+    when small tiles hold at least half of the elements (costa_debug_split)."""
     small = total = 0
-    tile_kernel = False
+    tile_kernel = patches = False
     for p, _, _, LA, LB in mats:
         t, pieces, _ = costa.costa_debug_split(LA, LB, p.op)
+        patches |= len(costa.costa_debug_patches(LA, LB, p.op)[0]) > 0
         if len(pieces):
             small += int((pieces["nx"].astype("int64") * pieces["ny"]).sum())
             tile_kernel |= len(t) > 0
         total += p.A.m * p.A.n
-    if len(mats) > 1 and 2 * small < total:
-        return "remap_kernel (direct)"
-    if small == 0:
-        return "remap_kernel (direct)"
-    return ("remap_kernel + " if tile_kernel else "") + "remap_small_kernel (direct)"
+    tiles = "remap_kernel"
+    if small and not (len(mats) > 1 and 2 * small < total):
+        tiles = ("remap_kernel + " if tile_kernel else "") + "remap_small_kernel"
+    return ("remap_patch_kernel or " if patches else "") + tiles + " (direct)"
 
 
 def message_phases(args, probs, stats, step, stream, dev):

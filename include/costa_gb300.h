@@ -486,8 +486,9 @@ costa_status costa_debug_axis_pieces(costa_layout A, costa_layout B, costa_op op
 
 /* Diagnostics (host only, no device work): the tile kernel's list for
  * (A, B, op) in direct mode, in the order the kernel's warps take the tiles
- * (pairs that run on patches move the same elements by those).  Each tile is 32 bytes: {source address, target
- * address (uint64), source stride, target stride (int32), nx, ny, problem,
+ * (pairs that run on patches move the same elements by those).  Each tile is
+ * 32 bytes: {source address, target address (uint64), source stride, target
+ * stride (int32), nx, ny, problem,
  * flags (uint16)}, in the frame where x runs along A's contiguous axis
  * (flags: 1 = transposed, 2 = vector path, 4 = conjugate).  Writes
  * min(*count, cap) tiles to out (32 * cap bytes) and the total to *count. */
@@ -549,12 +550,12 @@ costa_status costa_debug_exchange(costa_layout A, costa_layout B, costa_op op, i
  * mostly small, partial or misaligned, and large ones of 4- and 8-byte
  * elements.  A patch is a window of A's storage (at most
  * 32 x 32 elements, 16 x 16 for 16-byte elements; less for small matrices)
- * that may cover several overlay cells: 32 bytes {target address (uint64), target stride (int32),
+ * that may cover several overlay cells: 32 bytes {target address (uint64),
+ * target stride (int32),
  * first cell (uint32), lmask, rmask (uint32), nx, ny (uint8), problem, flags,
  * padding (uint16)}, x along A's contiguous axis.  The source is cut into
  * segments along the lane axis (the source's contiguous one: y when flags
- * has 1 = transposed, else x; 2: 4-byte source runs of whole aligned 16-byte
- * chunks) and the run axis (the other): bit k of lmask /
+ * has 1 = transposed, else x; 2: staged by whole aligned 16-byte chunks) and the run axis (the other): bit k of lmask /
  * rmask is set where one starts.  Segment pair (r, l) is cell first + r *
  * popcount(lmask) + l, 16 bytes {address (uint64), source stride (int32),
  * padding}: its element (run i, lane j of the patch) is at address +
