@@ -13,6 +13,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 
 import numpy as np
 
@@ -143,20 +144,21 @@ def _p(a: np.ndarray) -> int:
     return a.ctypes.data
 
 
-# Host arrays of the calls that run per transform are ctypes arrays made from
-# the caller's lists: 0.1 to 0.8 us each on the Grace host, where a numpy
+# Host arrays of the calls that run per transform are packed or ctypes arrays made
+# from the caller's lists: 0.1 to 0.8 us each on the Grace host, where a numpy
 # conversion and the array's address take 1.1 to 2 (the GPU's work is often
 # shorter than that).
-_DESC = ctypes.c_int64 * 9
+_DESC = struct.Struct("=9q")
 
 
 def _desc(desc):
-    """A ScaLAPACK array descriptor as a C array (anything but a list of nine
-    integers goes through numpy)."""
+    """A ScaLAPACK array descriptor as a C array.  Nine integers are packed
+    (which refuses values beyond 64 bits, where a ctypes array would wrap them);
+    anything else goes through numpy."""
     if isinstance(desc, (list, tuple)) and len(desc) == 9:
         try:
-            return _DESC(*desc)
-        except TypeError:
+            return _DESC.pack(*desc)
+        except struct.error:
             pass
     return _i64(desc).ctypes
 

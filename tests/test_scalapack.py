@@ -86,6 +86,43 @@ def test_submatrix_layout_validation():
 # GPU: pxgemr2d / pxtran against the oracle
 # ----------------------------------------------------------------------------
 
+@pytest.mark.parametrize("value", [2 ** 64 + 5, 2 ** 63, -(2 ** 63) - 1])
+@pytest.mark.parametrize("kind", [list, tuple])
+def test_descriptor_entries_beyond_64_bits_are_refused(value, kind):
+    """An entry that no 64-bit integer holds is refused, not wrapped: 2^64 + 5
+    would otherwise act as a block size of 5."""
+    c = rand_case(1)
+    g = _fake_grid(c, 8)
+    bad = kind(c["desc"][:4] + [value] + c["desc"][5:])
+    args = ("f64", c["m"], c["n"])
+    with pytest.raises(OverflowError):
+        costa.costa_pxgemr2d(*args, g, c["i"], c["j"], bad, g, c["i"], c["j"], c["desc"])
+    with pytest.raises(OverflowError):
+        costa.costa_pxgemr2d(*args, g, c["i"], c["j"], c["desc"], g, c["i"], c["j"], bad)
+    with pytest.raises(OverflowError):
+        costa.costa_pxtran(*args, 1.0, g, c["i"], c["j"], bad, 0.0, g, c["i"], c["j"], c["desc"])
+    with pytest.raises(OverflowError):
+        costa.costa_layout_create_scalapack("f64", g, c["i"], c["j"], c["m"], c["n"], bad)
+
+
+def test_descriptor_forms():
+    """Lists, tuples, numpy integers and floats, and arrays name the same
+    descriptor; the extremes of 64 bits are kept."""
+    from paper_2106_06601_gb300 import _desc
+
+    want = [1, 0, -(2 ** 63), 2 ** 63 - 1, 5, 6, 7, 8, 9]
+
+    def values(p):
+        import ctypes
+        if isinstance(p, bytes):
+            return list(np.frombuffer(p, np.int64))
+        return list((ctypes.c_int64 * 9).from_address(p.data))
+
+    for form in (want, tuple(want), [np.int64(v) for v in want], np.array(want, np.int64)):
+        assert values(_desc(form)) == want
+    assert values(_desc([1.0, 0, 30, 40, 5, np.int32(6), True, 8, 9])) == [1, 0, 30, 40, 5, 6, 1, 8, 9]
+
+
 def _matrix(c, dtype, dev, kind, seed, stream0):
     """A full ScaLAPACK matrix: one host and one device arena over the ranks'
     local matrices, plus the submatrix spec and the grid."""
