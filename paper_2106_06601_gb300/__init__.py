@@ -539,7 +539,9 @@ def costa_transform_batched(As, Bs, ops, alphas, betas, relabel: bool = False,
     handles = ctypes.c_void_p * n
     ha = handles(*[a.handle.value for a in As])
     hb = handles(*[b.handle.value for b in Bs])
-    op = (ctypes.c_int32 * n)(*[OPS[o] for o in ops])
+    codes = [OPS[o] for o in ops]
+    assert len(codes) >= n
+    op = (ctypes.c_int32 * len(codes))(*codes)
     al, be = _scalar_list(As[0].dtype, alphas, n), _scalar_list(As[0].dtype, betas, n)
     _check(_lib.costa_transform_batched_ex(n, ha, hb, op, al, be, relabel, out, MODES[mode], stream))
     return sigma

@@ -135,6 +135,20 @@ def test_transform_validation_before_device_work():
         L.destroy()
 
 
+def test_batch_lists_longer_and_shorter_than_the_batch():
+    """The ops of a batch may be more than its pairs (the first ones count, as
+    the library reads them); fewer are refused.  The shapes do not match, so
+    the call ends in validation, before any device work."""
+    p, q = C.c1(), C.fuzz_problem(3)
+    A = costa.costa_layout_from_spec(p.A, "f64", _spec_arrays(p.A))
+    B = costa.costa_layout_from_spec(q.B, "f64", _spec_arrays(q.B))
+    _expect(3, costa.costa_transform_batched, [A, A], [B, B], ["N", "T", "C"], [1.0, 1.0], [0.0, 0.0])
+    with pytest.raises(AssertionError):
+        costa.costa_transform_batched([A, A], [B, B], ["N"], [1.0, 1.0], [0.0, 0.0])
+    for L in (A, B):
+        L.destroy()
+
+
 # ----------------------------------------------------------------------------
 # relabeling (host Hungarian) against the oracle's exact solvers
 # ----------------------------------------------------------------------------
