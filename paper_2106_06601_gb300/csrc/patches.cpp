@@ -296,8 +296,11 @@ bool append_patches(const ProblemHost &ph, int prob, int64_t total, PatchList &o
     const bool aligned_ld = static_cast<int64_t>(B->blocks[0].ld) * es % 1024 == 0;
     const bool mix = lane_axis.shared * (transpose ? 350 : 1024) > lane_axis.extent * es && !(transpose && aligned_ld);
     const size_t chunk = mix ? 2 : longest;
-    for (size_t k0 = 0; k0 < longest; k0 += chunk)
-        for (size_t cy = 0; cy + 1 < Y.chain0.size(); ++cy) {
+    std::vector<size_t> live(Y.chain0.size() - 1);  // the chains with rows left, so that the work is one step per row
+    for (size_t cy = 0; cy < live.size(); ++cy) live[cy] = cy;
+    for (size_t k0 = 0; !live.empty(); k0 += chunk) {
+        size_t left = 0;
+        for (const size_t cy : live) {
             const size_t y0 = Y.chain0[cy] + k0, y1 = std::min(y0 + chunk, Y.chain0[cy + 1]);
             for (size_t cx = 0; cx + 1 < X.chain0.size(); ++cx)
                 for (size_t y = y0; y < y1; ++y) {
@@ -306,7 +309,10 @@ bool append_patches(const ProblemHost &ph, int prob, int64_t total, PatchList &o
                     patch0 += static_cast<int64_t>(x1 - x0);
                     cell0 += (X.nseg_sum[x1] - X.nseg_sum[x0]) * Y.patches[y].nseg;
                 }
+            if (y1 < Y.chain0[cy + 1]) live[left++] = cy;
         }
+        live.resize(left);
+    }
     out.patches.resize(out.patches.size() + static_cast<size_t>(npatches));
     out.cells.resize(out.cells.size() + static_cast<size_t>(ncells));
     const int64_t per_row = std::max<int64_t>(1, (npatches + ncells) / std::max<int64_t>(1, static_cast<int64_t>(work.size())));

@@ -145,3 +145,32 @@ def test_chunks_of_aligned_f32_runs(op, mb, ma, pad, chunks):
     patches, _ = costa.costa_debug_patches(LA, LB, op)
     share = np.mean((patches["flags"] & 2) != 0)
     assert share > 0.5 if chunks else share < 0.25
+
+
+def test_planning_time_of_one_long_chain_beside_many_short_ones():
+    """The order that mixes the chains' rows takes one step per row of
+    patches: a target of one wide block beside 60,000 single columns, over
+    16 single-row blocks (1.9 million patches), is planned in about a second,
+    not in the product of the three numbers of chains (3e10 steps)."""
+    import time
+
+    rows, wide, single = 16, 60000 * 32, 60000
+    cols = np.concatenate([[0, wide], wide + 1 + np.arange(single)])
+    nbc = single + 1
+    at = np.arange(rows * nbc, dtype=np.int64).reshape(rows, nbc)
+    one = np.ones((rows, nbc), np.int32)
+    LA = costa.costa_layout_create("f64", 1, np.arange(rows + 1), cols, 0 * one, FAKE + at * (1 << 26), one, 0 * one)
+    n = wide + single
+    LB = costa.costa_layout_create("f64", 1, np.array([0, rows]), np.array([0, n]), np.zeros((1, 1), np.int32),
+                                   np.array([[FAKE << 8]]), np.array([[rows + 1]]), np.zeros((1, 1), np.int32))
+    try:
+        t0 = time.perf_counter()
+        patches, cells = costa.costa_debug_patches(LA, LB, "N")
+        took = time.perf_counter() - t0
+    finally:
+        LA.destroy()
+        LB.destroy()
+    assert len(patches) == rows * (wide // 32 + single) == len(cells)
+    # mixed: two patches of the wide block's first row, then single columns
+    assert list(patches["ny"][:4]) == [32, 32, 32, 32] and patches["ny"][2 * rows] == 1
+    assert took < 12, took  # two calls of the planner; 0.9 s on an idle host
