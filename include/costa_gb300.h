@@ -53,10 +53,11 @@
  *    exactly rounded value: by the compensated dot product Dot2 (Ogita,
  *    Rump & Oishi 2005) for single-precision data; for double-precision
  *    data whose operands are all zero or of magnitude in [2^-480, 2^480),
- *    by an exact fixed-point sum on the integer pipes rounded once (every
- *    four-product component, the imaginary two-product ones) and by
- *    Kahan's algorithm for 2 x 2 determinants (the real two-product
- *    ones); Dot2 otherwise.  Repeated calls on one pair give the same
+ *    by a fixed-point sum on the integer pipes rounded once (four products:
+ *    within 0.5 ulp of the result plus 2^-5 ulp of the largest product) and
+ *    by Kahan's algorithm for 2 x 2 determinants or a fixed-point sum with
+ *    more bits (two products: within 2^-52 of the exact value, also where
+ *    they cancel); Dot2 otherwise.  Repeated calls on one pair give the same
  *    bits.  When beta == 0, A is never read, so NaN or garbage in
  *    A does not propagate.
  */
@@ -583,9 +584,10 @@ costa_status costa_debug_tma(costa_layout A, costa_layout B, costa_op op, int64_
  * that the remap kernels use for each component of alpha * op(B) + beta * A
  * with complex scalars on double complex data (Eq. 1), evaluated on the host
  * by the same code.  For each of `count` sets, out[k] = the sum over
- * i < n of (-1)^neg[k n + i] x[k n + i] * y[k n + i], rounded once to
- * double (within 0.5 ulp of the result plus n * 2^-7 ulp of the largest
- * product of the exact sum); n is 2 or 4.  x, y, neg, out: host arrays.
+ * i < n of (-1)^neg[k n + i] x[k n + i] * y[k n + i] in double, within 0.5 ulp
+ * of the result plus n * 2^-7 ulp of the largest product of the exact sum, and
+ * for n = 2 also within 2^-52 of the exact sum; n is 2 or 4.  x, y, neg, out:
+ * host arrays.
  * Every factor must be zero or of magnitude in [2^-480, 2^480), the range
  * in which the kernels take this evaluation; COSTA_ERR_INVALID_ARG
  * otherwise, with nothing written. */

@@ -1738,9 +1738,7 @@ costa_status costa_debug_fxdot(int n, int64_t count, const double *x, const doub
         const double *xk = x + k * n, *yk = y + k * n;
         const int32_t *nk = neg + k * n;
         if (n == 2) {
-            const fx::Term t[2] = {fx::mul(fx::unpack(xk[0]), fx::unpack(yk[0]), nk[0] ? 1u : 0u),
-                                   fx::mul(fx::unpack(xk[1]), fx::unpack(yk[1]), nk[1] ? 1u : 0u)};
-            out[k] = fx::sum<true>(t);  // as the kernels sum two products
+            out[k] = fx::dot2_mid(nk[0] ? -xk[0] : xk[0], yk[0], nk[1] ? -xk[1] : xk[1], yk[1]);
         } else {
             fx::Term t[4];
             for (int i = 0; i < 4; ++i) t[i] = fx::mul(fx::unpack(xk[i]), fx::unpack(yk[i]), nk[i] ? 1u : 0u);

@@ -135,15 +135,16 @@ enum : int32_t { SF_BETA0 = 1, SF_ALPHA1 = 2, SF_CPLX = 4, SF_BPOW2 = 8, SF_AREA
 //   K_SCALE real alpha, beta = 0       out = alpha * op(b)
 //   K_AXPBY real alpha, beta != 0      out = fma(alpha, op(b), beta * a)
 //   K_CPLX  complex beta (or complex alpha with beta != 0): each component
-//           a compensated sum of its four products (Dot2)
+//           a compensated sum of its four products (Dot2; double data in the
+//           middle range: fx::sum)
 //   K_CPLXR as K_CPLX for double complex data and a real alpha (SF_AREAL): the
 //            same bits without the two products that are zero
 //   K_AXPBY2 as K_AXPBY with beta = +-2^k: beta * a is formed exactly on the
 //            integer pipes (exponent add), saving one multiply on the scarce
 //            FP64 pipe; same bits as K_AXPBY
 //   K_CSCALE complex alpha, beta = 0   out = alpha * op(b) by Dot2 (double
-//            data in the middle range: Kahan's 2 x 2 determinant algorithm);
-//            A is not read (BLAS convention), so NaN in A does not propagate
+//            data in the middle range: Kahan's 2 x 2 determinant algorithm
+//            and fx::dot2_mid); A is not read (BLAS convention), so NaN in A does not propagate
 enum : int { K_COPY = 0, K_SCALE = 1, K_AXPBY = 2, K_CPLX = 3, K_AXPBY2 = 4, K_CSCALE = 5, K_CPLXR = 6, K_NKINDS = 7 };
 
 // The kinds whose output depends on A's old value (beta != 0).

@@ -15,10 +15,12 @@
 //      U = 2^-7 ulp(M) or finer (M the largest product): dropping and
 //      alignment together truncate less than one U per product;
 //   3. the integer sum is rounded once to double, to nearest even, by the
-//      hardware's conversion or on the integer pipes (the same bits), and the
+//      hardware's conversion (dot2_mid: with integer instructions), and the
 //      exponent added to its exponent field.
 // The result is within 0.5 ulp(x) + n U of the exact sum x of the n exact
-// products: n U <= 2^-5 ulp(M), so at most 0.5 ulp(x) + 0.032 ulp(M).  All
+// products: n U <= 2^-5 ulp(M), so at most 0.5 ulp(x) + 0.032 ulp(M).  Where
+// products cancel, that is far above an ulp of x; sums of two products, whose
+// alternative is Kahan's algorithm with 2u|x|, carry 32 bits more (dot2_mid).  All
 // intermediate magnitudes stay in the normal range: a product lies in
 // [2^-960, 2^960), the sum below 2^962, and a nonzero result is a multiple of
 // U >= 2^-1019.
@@ -35,13 +37,16 @@
 // arithmetic can be checked without a GPU.
 #pragma once
 
+#include <cmath>
 #include <cstdint>
 #include <cstring>
 
 #ifdef __CUDACC__
 #define COSTA_FX_HD __host__ __device__ __forceinline__
+#define COSTA_FX_HD_CALL static __host__ __device__ __noinline__
 #else
 #define COSTA_FX_HD inline
+#define COSTA_FX_HD_CALL inline
 #endif
 
 namespace costa {
@@ -100,19 +105,6 @@ COSTA_FX_HD double round_to_double(int64_t v) {
 #endif
 }
 
-// The same, |v| < 2^63, without the conversion, for the complex-alpha kind: its
-// other component is formed on the FP64 pipe, and the conversions' rate is as
-// low.  GB300, c128 BC64 -> BC128 T, complex alpha, us per call, conversion ->
-// this: 2048^2 56.2 -> 49.6, 4096^2 173.0 -> 147.9; but with a complex beta, one
-// component of two so, 233 -> 256 (the ALU pipe bounds it).
-COSTA_FX_HD uint64_t round_to_double_bits_alu(int64_t v) {
-    const uint64_t neg = static_cast<uint64_t>(v >> 63), mag = (static_cast<uint64_t>(v) ^ neg) - neg;
-    const uint32_t lz = leading_zeros(mag | 1u);  // >= 1
-    const uint64_t m = mag << (lz - 1u);        // leading bit at 62
-    const uint64_t q = (m + 0x1FFu + ((m >> 10) & 1u)) >> 10;  // 53 bits, ties to even; a carry moves on to the exponent
-    return (neg << 63) + ((static_cast<uint64_t>(1085u - lz) << 52) + q);
-}
-
 // An operand: its 53-bit significand as 31 top bits (h) and 22 low bits at the
 // top of a word (l = low bits * 2^10), both 0 for a zero; its biased exponent (kZeroExp for a zero, so that a zero
 // product never is the largest); its sign as a mask.
@@ -145,10 +137,11 @@ COSTA_FX_HD Op unpack(double v) {
 }
 
 // One product x * y, negated when neg = 1: floor(significand product / 2^44)
-// (in [2^60, 2^62), or 0), the sum of the biased exponents and the sign as a
-// mask.
+// (in [2^60, 2^62), or 0), the next 32 bits of that quotient, the sum of the
+// biased exponents and the sign as a mask.
 struct Term {
     uint64_t p;
+    uint32_t r;
     int32_t e;
     uint32_t s;
 };
@@ -158,14 +151,21 @@ COSTA_FX_HD Term mul(const Op &x, const Op &y, uint32_t neg) {
     const uint64_t low = mad_wide(x.l, y.l, 0) >> 32;
     const uint64_t mid = mad_wide(x.l, y.h, mad_wide(x.h, y.l, low));  // below 2^64 (h < 2^31)
     t.p = mad_wide(x.h, y.h, mid >> 32);
+    t.r = static_cast<uint32_t>(mid);
     t.e = x.e + y.e;
     t.s = x.s ^ y.s ^ (neg ? 0xFFFFFFFFu : 0u);
     return t;
 }
 
+// bits * 2^(emax - 2105) for the bits of a nonzero double: a sum's unit (a
+// significand product has unit 2^(emax - 2150), and this is 2^45 of it).
+COSTA_FX_HD double scaled(uint64_t bits, int32_t emax) {
+    return from_bits(bits + (static_cast<uint64_t>(static_cast<int64_t>(emax - 2105)) << 52));
+}
+
 // The sum of n <= 4 terms, rounded once to double (to nearest, ties to even).
-// A zero sum gives +0.  ALU: rounded without the hardware's conversion.
-template <bool ALU = false, int N>
+// A zero sum gives +0.
+template <int N>
 COSTA_FX_HD double sum(const Term (&t)[N]) {
     int32_t emax = t[0].e;
 #pragma unroll
@@ -181,11 +181,99 @@ COSTA_FX_HD double sum(const Term (&t)[N]) {
     }
     acc -= static_cast<uint64_t>(static_cast<int64_t>(static_cast<int32_t>(neg)));
     if (acc == 0) return 0.0;
-    // acc's unit is 2^(emax - 2105): a significand product has unit
-    // 2^(emax - 2150), and acc's is 2^45 of it
-    const uint64_t r = ALU ? round_to_double_bits_alu(static_cast<int64_t>(acc))
-                           : bits_of(round_to_double(static_cast<int64_t>(acc)));
-    return from_bits(r + (static_cast<uint64_t>(static_cast<int64_t>(emax - 2105)) << 52));
+    return scaled(bits_of(round_to_double(static_cast<int64_t>(acc))), emax);
+}
+
+// ---- sums of two products ----
+
+COSTA_FX_HD double fma_rn(double x, double y, double z) {
+#ifdef __CUDA_ARCH__
+    return __fma_rn(x, y, z);
+#else
+    return std::fma(x, y, z);
+#endif
+}
+COSTA_FX_HD double mul_rn(double x, double y) {
+#ifdef __CUDA_ARCH__
+    return __dmul_rn(x, y);
+#else
+    return x * y;
+#endif
+}
+COSTA_FX_HD double add_rn(double x, double y) {
+#ifdef __CUDA_ARCH__
+    return __dadd_rn(x, y);
+#else
+    return x + y;
+#endif
+}
+
+// x * y + z * t, or x * y - z * t (minus), with Kahan's algorithm for 2 x 2
+// determinants: w = z * t rounded, its error e exactly by one fma, then (x * y
+// +- w) rounded by a second fma and +- e added.  Jeannerod, Louvet and Muller
+// ("Further analysis of Kahan's algorithm for the accurate computation of
+// 2 x 2 determinants", Math. Comp. 82, 2013) bound its error by 2u|exact|
+// when nothing overflows or underflows: within 2 ulps of the exact value,
+// and so of the oracle's compensated result.  4 FP64 operations instead of
+// Dot2's 13.
+COSTA_FX_HD double kahan2(double x, double y, double z, double t, bool minus) {
+    const double w = mul_rn(z, t);
+    const double e = fma_rn(z, t, -w);  // z * t = w + e exactly
+    return minus ? add_rn(fma_rn(x, y, -w), -e) : add_rn(fma_rn(x, y, w), e);
+}
+
+// A call of its own, so that the FP64 pipe is not held by instructions that are
+// predicated off.
+COSTA_FX_HD_CALL double kahan2_far(double x, double y, double z, double t) { return kahan2(x, y, z, t, false); }
+
+// The low 32 bits of (hi:lo) >> n, hi for n >= 32; the high 32 of (hi:lo) << n, n < 32.
+COSTA_FX_HD uint32_t funnel_shr(uint32_t lo, uint32_t hi, uint32_t n) {
+#ifdef __CUDA_ARCH__
+    return __funnelshift_rc(lo, hi, n);
+#else
+    return n < 32u ? static_cast<uint32_t>(((static_cast<uint64_t>(hi) << 32) | lo) >> n) : hi;
+#endif
+}
+COSTA_FX_HD uint32_t funnel_shl(uint32_t lo, uint32_t hi, uint32_t n) {
+#ifdef __CUDA_ARCH__
+    return __funnelshift_l(lo, hi, n);
+#else
+    return static_cast<uint32_t>(((static_cast<uint64_t>(hi) << 32 | lo) << n) >> 32);
+#endif
+}
+
+// x * y + z * t for operands in range, within 2u of the exact value (u =
+// 2^-53), the bound of Kahan's algorithm, whatever cancels: a sum in fixed
+// point with 32 bits more than `sum` has, so that it is within 1.02u wherever
+// it has at least 2^31 of sum's units (the larger product has at least 2^59):
+// terms of nearly the same exponent are off by less than 2^-32 of a unit each;
+// one that is shifted by more than 32 bits is off by less than a unit, but
+// then nothing cancels.  Below, Kahan's algorithm.  Rounded without the
+// hardware's conversion: the other component of the complex-alpha kind is
+// formed on the FP64 pipe, and the conversions' rate is as low (without the 32
+// bits 173 -> 148 us).  GB300, c128 4096^2 T, complex alpha, BC64 -> BC128, us
+// per call: 157; Kahan's algorithm for both components 212; no more bits than
+// `sum`, and Kahan's algorithm below 2^54 units (a third of the warps) 173;
+// never Kahan's algorithm, thousands of ulps off where the products cancel, 148.
+COSTA_FX_HD double dot2_mid(double x, double y, double z, double t) {
+    const Term a = mul(unpack(x), unpack(y), 0u), b = mul(unpack(z), unpack(t), 0u);
+    const int32_t emax = a.e > b.e ? a.e : b.e;
+    const uint32_t na = static_cast<uint32_t>(emax - a.e + 1), nb = static_cast<uint32_t>(emax - b.e + 1);
+    // two's complement, the 32 bits below the unit in `low`
+    const uint64_t low = static_cast<uint64_t>(funnel_shr(a.r, static_cast<uint32_t>(a.p), na) ^ a.s) +
+                         (funnel_shr(b.r, static_cast<uint32_t>(b.p), nb) ^ b.s) + ((a.s & 1u) + (b.s & 1u));
+    const uint64_t acc = (shr_clamp(a.p, na) ^ (static_cast<uint64_t>(a.s) << 32 | a.s)) +
+                         (shr_clamp(b.p, nb) ^ (static_cast<uint64_t>(b.s) << 32 | b.s)) + (low >> 32);
+    const uint32_t sgn = static_cast<uint32_t>(static_cast<int64_t>(acc) >> 63);
+    const uint64_t rest = static_cast<uint64_t>(static_cast<uint32_t>(low) ^ sgn) + (sgn & 1u);
+    const uint64_t mag = (acc ^ (static_cast<uint64_t>(sgn) << 32 | sgn)) + (rest >> 32);
+    if (mag < (uint64_t(1) << 31)) return (a.p | b.p) ? kahan2_far(x, y, z, t) : 0.0;
+    const uint32_t lz = leading_zeros(mag), up = lz - 1u;  // up < 32
+    const uint32_t mid = static_cast<uint32_t>(mag);
+    const uint64_t m = static_cast<uint64_t>(funnel_shl(mid, static_cast<uint32_t>(mag >> 32), up)) << 32 |
+                       funnel_shl(static_cast<uint32_t>(rest), mid, up);  // leading bit at 62
+    const uint64_t q = (m + 0x1FFu + ((m >> 10) & 1u)) >> 10;  // 53 bits, ties to even; a carry moves on to the exponent
+    return scaled((static_cast<uint64_t>(sgn) << 63) + (static_cast<uint64_t>(1085u - lz) << 52) + q, emax);
 }
 
 }  // namespace fx

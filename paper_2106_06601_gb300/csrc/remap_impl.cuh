@@ -30,8 +30,8 @@
 //
 // "alpha and beta as one fma" holds for real scalars; complex scalars take
 // a compensated evaluation per component (Dot2; for double data Kahan's
-// algorithm when a component has two terms, and a fixed-point sum on the
-// integer pipes when it has four), see combine_c.
+// algorithm or a fixed-point sum on the integer pipes when a component has two
+// terms, and a fixed-point sum when it has four), see combine_c.
 //
 // The kernel walks a list of tile descriptors (TileDesc) resolved on the host:
 // the direct list (every tile: B -> A), or the message path of Alg. 3 /
@@ -97,8 +97,9 @@ template <> struct ET<double2> { enum { VEC = 1, CPLX = 1 }; typedef double R; }
 //    with Kahan's algorithm alone): T and N 1458 -> 2133 with 2 to 4
 //    blocks; with half of the components summed in fixed point on the integer
 //    pipes, unrolled, 2557 at 2 blocks, 2660 at 3 (a third or a quarter of
-//    them: 2553, 2569); in the rolled loop, 3 blocks, 3259; with their
-//    imaginary components' sums rounded on the integer pipes too, 3630.
+//    them: 2553, 2569); in the rolled loop, 3 blocks, 3259; with the
+//    imaginary components in fixed point, rounded on the integer pipes too,
+//    3420 (fx::dot2_mid).
 //  - c64 complex scalars, against 3 blocks with 2 buffers: complex beta
 //    T 4484 -> 5482, N 4495 -> 5495 with 4 blocks and no look-ahead;
 //    complex alpha T 5551 -> 5955 with two tiles ahead; the real general
@@ -446,20 +447,6 @@ __device__ __forceinline__ bool mid_range(double v) {
     return (((hi & 0x7FFFFFFFu) | lo) == 0u) || (e - (1023u - 480u)) < 960u;
 }
 
-// x * y + sgn * (z * t) with Kahan's algorithm for 2 x 2 determinants: w =
-// z * t rounded, its error e exactly by one fma, then (x * y + sgn * w)
-// rounded by a second fma and sgn * e added.  Jeannerod, Louvet and Muller
-// ("Further analysis of Kahan's algorithm for the accurate computation of
-// 2 x 2 determinants", Math. Comp. 82, 2013) bound its error by 2u|exact|
-// when nothing overflows or underflows: within 2 ulps of the exact value,
-// and so of the oracle's compensated result.  4 FP64 operations instead of
-// Dot2's 13.
-__device__ __forceinline__ double kahan2(double x, double y, double z, double t, bool minus) {
-    const double w = __dmul_rn(z, t);
-    const double e = __fma_rn(z, t, -w);  // z * t = w + e exactly
-    return minus ? __dsub_rn(__fma_rn(x, y, -w), e) : __dadd_rn(__fma_rn(x, y, w), e);
-}
-
 // Passes of a tile that the drain of double complex data with complex
 // scalars evaluates together (stage_drain).
 #ifndef COSTA_FX_GROUP
@@ -505,16 +492,14 @@ __device__ __forceinline__ double2 fx_cplx(const double2 &b, const double2 &a, c
 
 // alpha * b for double complex data and a complex alpha, every operand in the
 // middle range: the real component by Kahan's algorithm on the FP64 pipe, the
-// imaginary one as a fixed-point sum on the integer pipes (fxdot.h), so that
-// both pipes work.  The choice depends on nothing but the component, so every
-// kernel and work list gives the same bits.
+// imaginary one on the integer pipes (fx::dot2_mid), so that both pipes work.
+// Both are within 2u of the exact component, whatever cancels.  The choice
+// depends on nothing but the component, so every kernel and work list gives the
+// same bits.
 __device__ __forceinline__ double2 mid_cscale(const double2 &b, const Sc &s) {
-    const fx::Op fbx = fx::unpack(b.x), fby = fx::unpack(b.y);
-    const fx::Op far = fx::unpack(s.ar), fai = fx::unpack(s.ai);
-    const fx::Term im[2] = {fx::mul(far, fby, 0u), fx::mul(fai, fbx, 0u)};  // ar by + ai bx
     double2 o;
-    o.x = kahan2(s.ar, b.x, s.ai, b.y, true);  // ar bx - ai by
-    o.y = fx::sum<true>(im);
+    o.x = fx::kahan2(s.ar, b.x, s.ai, b.y, true);  // ar bx - ai by
+    o.y = fx::dot2_mid(s.ar, b.y, s.ai, b.x);      // ar by + ai bx
     return o;
 }
 

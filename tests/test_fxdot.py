@@ -63,6 +63,35 @@ def test_fxdot_within_its_bound_of_the_exact_sum(n):
         assert abs(Fraction(float(got[k])) - exact) <= bound, (k, x[k], y[k], neg[k], got[k], rounded)
 
 
+def test_two_products_that_cancel_keep_their_relative_accuracy():
+    """Sums of two products are within 2u of the exact value (u = 2^-53), the
+    bound of Kahan's algorithm for 2 x 2 determinants, whatever cancels: the
+    second product is set against the first to 0 to 60 bits, exactly, and
+    about the size where the evaluation changes (a sum of 2^-5 of the larger
+    product)."""
+    rng = random.Random(31)
+    x, y = [], []
+    for k in range(24000):
+        a, b, c = (rng.choice([-1, 1]) * rng.uniform(0.5, 1) * 2.0 ** rng.randint(-40, 40) for _ in range(3))
+        bits = rng.choice([rng.randint(0, 60), 5, 6, 7, 200])
+        d = -(a * b / c) * (1 + rng.choice([-1, 1]) * rng.uniform(0.5, 1) * 2.0 ** -bits)
+        x.append((a, c))
+        y.append((b, d))
+    x, y = np.array(x), np.array(y)
+    got = costa.costa_debug_fxdot(x, y, np.zeros(x.shape, np.int32))
+    worst, square = Fraction(0), 0.0
+    for k in range(len(x)):
+        exact = Fraction(x[k, 0]) * Fraction(y[k, 0]) + Fraction(x[k, 1]) * Fraction(y[k, 1])
+        if exact == 0:
+            assert got[k] == 0.0
+            continue
+        err = abs((Fraction(float(got[k])) - exact) / exact)
+        worst = max(worst, err)
+        square += float(err) ** 2
+    assert worst <= Fraction(2, 2 ** 53), float(worst * 2 ** 53)
+    assert (square / len(x)) ** 0.5 <= 2.0 ** -53  # Kahan's own on these: about 0.6u
+
+
 def test_fxdot_closed_forms():
     t = 2.0 ** -27
     cases = [

@@ -408,6 +408,45 @@ def test_complex_scalars_within_2ulp(dtype, op, alpha, beta, dev):
             g.close()
 
 
+@pytest.mark.parametrize("op", ["N", "T", "C"])
+@pytest.mark.parametrize("mode", ["direct", "message"])
+def test_complex_alpha_keeps_relative_accuracy(op, mode, dev):
+    """alpha * op(b) for double complex data: both components within 2u of
+    their exact values (u = 2^-53, the bound of Kahan's algorithm), also where
+    their two products cancel to 0 to 60 bits, in every kernel."""
+    from fractions import Fraction
+
+    from tests._util import global_matrix, op_apply, scatter_global
+    alpha = complex(0.3, -0.4)
+    for k, (B, A) in enumerate(_complex_layouts(op)):
+        p = C.Problem("cancel", "c128", op, alpha, 0.0, A, B, "uniform", "nan", C.SEED0 + 60 + k)
+        g = OnDevice(p, dev)
+        try:
+            rng = np.random.default_rng(60 + k)
+            X = global_matrix(p.B, g.Bh.buffers())
+            re, im = X.real.ravel().copy(), X.imag.ravel().copy()
+            near = 1 + 2.0 ** -rng.integers(0, 61, re.size) * rng.uniform(0.5, 1, re.size)
+            sign = -1.0 if op == "C" else 1.0  # of b's imaginary part in op(b)
+            third = re.size // 3
+            im[:third] = (sign * alpha.real / alpha.imag * re * near)[:third]  # the real component cancels
+            im[-third:] = (-sign * alpha.imag / alpha.real * re * near)[-third:]  # the imaginary one
+            X = (re + 1j * im).reshape(X.shape)
+            scatter_global(p.B, g.Bh.buffers(), X)
+            g.Bd.upload(g.Bh)
+            g.run(mode=mode)
+            got = global_matrix(p.A, g.Ad.download().buffers()).ravel()
+            ar, ai = Fraction(alpha.real), Fraction(alpha.imag)
+            worst = Fraction(0)
+            for v, b in zip(got, op_apply(op, X).ravel()):
+                br, bi = Fraction(float(b.real)), Fraction(float(b.imag))
+                for have, exact in ((v.real, ar * br - ai * bi), (v.imag, ar * bi + ai * br)):
+                    err = abs(Fraction(float(have)) - exact)
+                    worst = max(worst, err / abs(exact) if exact else err)
+            assert worst <= Fraction(2, 2 ** 53), float(worst * 2 ** 53)
+        finally:
+            g.close()
+
+
 @pytest.mark.parametrize("dtype", ["c64", "c128"])
 @pytest.mark.parametrize("alpha,beta", [(complex(-0.6, 0.3), 0.0), (complex(0.2, 0.9), complex(-1.1, 0.4))])
 def test_special_values_complex_scalars(dtype, alpha, beta, dev):
