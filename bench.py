@@ -30,6 +30,7 @@ from __future__ import annotations
 import argparse
 import hashlib
 import json
+import math
 import os
 import platform
 import statistics
@@ -614,23 +615,27 @@ def run_e2e(args, costa, mats, step, stream, dev, world, nbytes):
 
 
 def direct_kernels(costa, mats):
-    """Which remap kernels the direct list may run: patches where the pairs
-    have them and the planner's rule for their type, size and scalars takes
-    them (costa_debug_patches), else the tile kernel, and the small-tile kernel
-    when small tiles hold at least half of the elements (costa_debug_split)."""
-    small = total = 0
-    tile_kernel = patches = False
-    for p, _, _, LA, LB in mats:
-        t, pieces, _ = costa.costa_debug_split(LA, LB, p.op)
-        patches |= len(costa.costa_debug_patches(LA, LB, p.op)[0]) > 0
-        if len(pieces):
-            small += int((pieces["nx"].astype("int64") * pieces["ny"]).sum())
-            tile_kernel |= len(t) > 0
-        total += p.A.m * p.A.n
-    tiles = "remap_kernel"
-    if small and not (len(mats) > 1 and 2 * small < total):
-        tiles = ("remap_kernel + " if tile_kernel else "") + "remap_small_kernel"
-    return ("remap_patch_kernel or " if patches else "") + tiles + " (direct)"
+    """The remap kernels that the direct call launches, from the planner's own
+    choice of work lists (costa_debug_dispatch)."""
+    d = costa.costa_debug_dispatch([m[3] for m in mats], [m[4] for m in mats], [m[0].op for m in mats])
+    patched = [combine_kind(p) in d["patch_kinds"] for p, *_ in mats]
+    names = ["remap_patch_kernel"] if any(patched) else []
+    if d["tiles_are_rest"] or not all(patched):
+        tma = any(combine_kind(p) in d["tma_kinds"] for p, *_ in mats)
+        names += ["remap_tma_kernel + remap_kernel"] if d["tiles"] and tma else ["remap_kernel"] if d["tiles"] else []
+        names += ["remap_kernel (misaligned)"] if d["misaligned"] else []
+        names += ["remap_small_kernel"] if d["pieces"] else []
+    return " + ".join(names) + " (direct)"
+
+
+def combine_kind(p):
+    """The combine kind of a problem's scalars, as costa_debug_dispatch names it."""
+    al, be = complex(p.alpha), complex(p.beta)
+    if al.imag or be.imag:
+        return "cscale" if be == 0 else "cplxr" if p.dtype == "c128" and not al.imag else "cplx"
+    if be == 0:
+        return "copy" if al == 1 else "scale"
+    return "axpby2" if math.frexp(abs(be.real))[0] == 0.5 else "axpby"
 
 
 def message_phases(args, probs, stats, step, stream, dev):

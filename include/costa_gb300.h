@@ -498,7 +498,7 @@ costa_status costa_debug_tiles(costa_layout A, costa_layout B, costa_op op, void
 
 /* Diagnostics (host only, no device work): how the direct tile list of
  * (A, B, op) is split between the tile kernel and the small-tile kernel, for
- * pairs that do not run on patches (costa_debug_patches).  Tiles needing fewer
+ * pairs that do not run on patches (costa_debug_dispatch).  Tiles needing fewer
  * than half of a full tile's warp passes are cut into pieces of one warp
  * pass each (at most 8 x 8 elements; 16 x 8 for 4-byte and 8 x 4 for
  * 16-byte elements, x along A's contiguous axis), which the small-tile
@@ -562,9 +562,24 @@ costa_status costa_debug_exchange(costa_layout A, costa_layout B, costa_op op, i
  * padding}: its element (run i, lane j of the patch) is at address +
  * (i * stride + j) elements.  Writes up to cap_patches patches and cap_cells
  * cells and the totals; 0 when the pair has no patches (layouts that mix
- * element orders). */
+ * element orders).  Whether a call runs on them is the planner's choice
+ * (costa_debug_dispatch). */
 costa_status costa_debug_patches(costa_layout A, costa_layout B, costa_op op, void *patches, int64_t cap_patches,
                                  void *cells, int64_t cap_cells, int64_t *npatches, int64_t *ncells);
+
+/* Diagnostics (host only, no device work): the work lists that direct calls
+ * of this batch run, by the planner's own rule.  out: host, 10 int64: the
+ * combine kinds that run on patches (bit per kind: 0 copy, 1 real alpha with
+ * beta = 0, 2 real scalars, 3 complex scalars with beta != 0, 4 real scalars
+ * with beta = +-2^k, 5 complex alpha with beta = 0, 6 complex beta with a real
+ * alpha on double complex data), the patches, their cells, 1 when the tiles
+ * are other problems' than the patches' (every kind runs on both lists) or 0
+ * when they are the same problems' for the kinds that do not run on patches,
+ * then the tiles, the misaligned tiles, the small pieces, the x-halves (cut
+ * into more where a list is short), and the kinds whose tiles and whose
+ * x-halves TMA may stage.  ops: host, n values. */
+costa_status costa_debug_dispatch(int n, const costa_layout *A, const costa_layout *B, const costa_op *ops,
+                                  int64_t *out);
 
 /* Diagnostics: TMA staging of the tile kernel's source tiles.  By default
  * (environment variable COSTA_TMA unset when a plan is built) only f64 data

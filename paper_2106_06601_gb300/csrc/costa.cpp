@@ -577,6 +577,71 @@ uint32_t take_patches(const Plan &plan, std::vector<TileDesc> &list, PatchList &
     return kAlignedPatchKinds | (4 * boxes < 3 * all ? 1u << K_AXPBY : 0u);
 }
 
+ProblemHost make_problem(const costa_layout_s *A, const costa_layout_s *B, costa_op op, int ts) {
+    ProblemHost ph;
+    ph.A = A;
+    ph.B = B;
+    ph.op = op;
+    ph.rows = cut_pair_axis(A, B, op, 0, ts);
+    ph.cols = cut_pair_axis(A, B, op, 1, ts);
+    return ph;
+}
+
+// The work lists of a plan's direct calls, on the host.
+struct DirectLists {
+    PatchList patches;
+    uint32_t patch_kinds = 0;  // the kinds that run on the patches
+    bool rest = true;          // the tiles are other problems' than the patches'
+    SplitList split;
+    std::vector<TileDesc> halves;
+    bool had_halves = false;
+    uint32_t tma_big = 0, tma_halves = 0;  // the kinds whose tiles TMA may stage
+};
+
+// Cuts the plan's problems into the lists that its direct calls run.
+costa_status direct_lists(const Plan &plan, DirectLists &out) {
+    const int n = static_cast<int>(plan.probs.size()), es = plan.esize, ts = plan.ts;
+    // the direct tile list, in (problem, row piece, column piece) order
+    std::vector<TileDesc> list;
+    if (n == 1) {
+        append_direct_tiles(plan.probs[0], 0, es, ts, list, false);  // ordered below, if the tiles are kept
+    } else {  // a batch: problems in parallel, each into its own range
+        std::vector<int64_t> start(static_cast<size_t>(n) + 1, 0);
+        for (int k = 0; k < n; ++k)
+            start[k + 1] = start[k] + static_cast<int64_t>(plan.probs[k].rows.tiles.size()) *
+                                          static_cast<int64_t>(plan.probs[k].cols.tiles.size());
+        list.resize(static_cast<size_t>(start[n]));
+        parallel_for(n, std::max<int64_t>(1, (int64_t(1) << 15) * n / std::max<int64_t>(1, start[n])),
+                     [&](int64_t k0, int64_t k1) {
+                         for (int64_t k = k0; k < k1; ++k) {
+                             std::vector<TileDesc> part;
+                             append_direct_tiles(plan.probs[k], static_cast<int>(k), es, ts, part);
+                             std::copy(part.begin(), part.end(), list.begin() + start[k]);
+                         }
+                     });
+    }
+    const costa_status st = check_extents(list, es, "direct");
+    if (st != COSTA_OK) return st;
+    const bool cplx = plan.dtype == COSTA_C64 || plan.dtype == COSTA_C128;
+    out.patch_kinds = take_patches(plan, list, out.patches, out.rest);
+    if (n == 1) order_direct_tiles(plan.probs[0], list, 0, es, ts);
+    out.split = split_small(std::move(list), es, cplx);
+    // The aligned tiles also as x-halves (see use_halves), for the kinds
+    // that run on them (see launch_list in transform_impl).
+    std::vector<char> halve(static_cast<size_t>(n), 0);
+    const bool any = out.rest || es == 4 || !((out.patch_kinds >> K_AXPBY2) & 1u);
+    for (int k = 0; k < n; ++k) halve[k] = any && use_halves(plan.probs[k], es);
+    out.halves = split_x_halves(out.split.big, ts / 2, es, halve);
+    out.had_halves = !out.halves.empty();
+    out.split.big = cut_few(std::move(out.split.big), es);
+    out.halves = cut_few(std::move(out.halves), es);
+    // TMA staging (tma.cpp): the kinds the policy would give it; their lists
+    // are built by the first call of such a kind (ensure_tma)
+    out.tma_big = tma_policy_kinds(out.split.big, es, cplx, false);
+    out.tma_halves = out.had_halves ? tma_policy_kinds(out.halves, es, cplx, true) : 0;
+    return COSTA_OK;
+}
+
 // Builds the overlay, the tile list and the device tables, and runs the
 // volume kernel.
 costa_status build_plan(int n, const costa_layout *As, const costa_layout *Bs, const costa_op *ops,
@@ -596,19 +661,14 @@ costa_status build_plan(int n, const costa_layout *As, const costa_layout *Bs, c
     plan->esize = esize_of(plan->dtype);
     plan->P = As[0]->nranks;
     plan->ts = tile_extent(plan->esize);
-    const int P = plan->P, ts = plan->ts, es = plan->esize;
+    const int P = plan->P, ts = plan->ts;
 
     Arena arena;
     struct Off { size_t irows, icols, ownA, ownB; };
     std::vector<Off> offs(n);
     int64_t tiles = 0, cells = 0;
     for (int k = 0; k < n; ++k) {
-        ProblemHost ph;
-        ph.A = As[k];
-        ph.B = Bs[k];
-        ph.op = ops[k];
-        ph.rows = cut_pair_axis(ph.A, ph.B, ph.op, 0, ts);
-        ph.cols = cut_pair_axis(ph.A, ph.B, ph.op, 1, ts);
+        ProblemHost ph = make_problem(As[k], Bs[k], ops[k], ts);
         Off &o = offs[k];
         o.irows = arena.add_vec(ph.rows.intervals);
         o.icols = arena.add_vec(ph.cols.intervals);
@@ -618,47 +678,14 @@ costa_status build_plan(int n, const costa_layout *As, const costa_layout *Bs, c
         cells += static_cast<int64_t>(ph.rows.intervals.size()) * static_cast<int64_t>(ph.cols.intervals.size());
         plan->probs.push_back(std::move(ph));
     }
-    // the direct tile list, in (problem, row piece, column piece) order
-    std::vector<TileDesc> list;
-    if (n == 1) {
-        append_direct_tiles(plan->probs[0], 0, es, ts, list, false);  // ordered below, if the tiles are kept
-    } else {  // a batch: problems in parallel, each into its own range
-        std::vector<int64_t> start(static_cast<size_t>(n) + 1, 0);
-        for (int k = 0; k < n; ++k)
-            start[k + 1] = start[k] + static_cast<int64_t>(plan->probs[k].rows.tiles.size()) *
-                                          static_cast<int64_t>(plan->probs[k].cols.tiles.size());
-        list.resize(static_cast<size_t>(start[n]));
-        parallel_for(n, std::max<int64_t>(1, (int64_t(1) << 15) * n / std::max<int64_t>(1, start[n])),
-                     [&](int64_t k0, int64_t k1) {
-                         for (int64_t k = k0; k < k1; ++k) {
-                             std::vector<TileDesc> part;
-                             append_direct_tiles(plan->probs[k], static_cast<int>(k), es, ts, part);
-                             std::copy(part.begin(), part.end(), list.begin() + start[k]);
-                         }
-                     });
-    }
-    {
-        costa_status st = check_extents(list, es, "direct");
-        if (st != COSTA_OK) return st;
-    }
-    const bool cplx = plan->dtype == COSTA_C64 || plan->dtype == COSTA_C128;
-    PatchList patches;
-    bool rest = true;
-    const uint32_t patch_kinds = take_patches(*plan, list, patches, rest);
-    if (n == 1) order_direct_tiles(plan->probs[0], list, 0, es, ts);
-    SplitList split = split_small(std::move(list), es, cplx);
-    // The aligned tiles also as x-halves (see use_halves), for the kinds
-    // that run on them (see launch_list in transform_impl).
-    std::vector<char> halve(static_cast<size_t>(n), 0);
-    for (int k = 0; k < n; ++k) halve[k] = (rest || es == 4 || !((patch_kinds >> K_AXPBY2) & 1u)) && use_halves(plan->probs[k], es);
-    std::vector<TileDesc> halves = split_x_halves(split.big, ts / 2, es, halve);
-    const bool had_halves = !halves.empty();
-    split.big = cut_few(std::move(split.big), es);
-    halves = cut_few(std::move(halves), es);
-    // TMA staging (tma.cpp): the kinds the policy would give it; their lists
-    // are built by the first call of such a kind (ensure_tma)
-    plan->tma_kinds_big = tma_policy_kinds(split.big, es, cplx, false);
-    plan->tma_kinds_halves = had_halves ? tma_policy_kinds(halves, es, cplx, true) : 0;
+    DirectLists lists;
+    costa_status st = direct_lists(*plan, lists);
+    if (st != COSTA_OK) return st;
+    const SplitList &split = lists.split;
+    const std::vector<TileDesc> &halves = lists.halves;
+    const PatchList &patches = lists.patches;
+    plan->tma_kinds_big = lists.tma_big;
+    plan->tma_kinds_halves = lists.tma_halves;
     const SplitOffsets off_tiles = arena.add_split(split);
     const size_t off_halves = halves.empty() ? 0 : arena.add_vec(halves);
     const size_t off_patches = arena.add_vec(patches.patches), off_pcells = arena.add_vec(patches.cells);
@@ -702,10 +729,10 @@ costa_status build_plan(int n, const costa_layout *As, const costa_layout *Bs, c
     plan->direct.patches = reinterpret_cast<const PatchDesc *>(dbase + off_patches);
     plan->direct.cells = reinterpret_cast<const PatchCell *>(dbase + off_pcells);
     plan->direct.npatches = static_cast<int64_t>(patches.patches.size());
-    plan->direct.patch_kinds = patch_kinds;
-    plan->direct.tiles_are_rest = rest;
+    plan->direct.patch_kinds = lists.patch_kinds;
+    plan->direct.tiles_are_rest = lists.rest;
     plan->direct_halves = plan->direct;
-    if (had_halves) {
+    if (lists.had_halves) {
         plan->direct_halves.tiles = reinterpret_cast<const TileDesc *>(dbase + off_halves);
         plan->direct_halves.ntiles = static_cast<int64_t>(halves.size());
     }
@@ -1702,6 +1729,31 @@ costa_status costa_debug_patches(costa_layout A, costa_layout B, costa_op op, vo
     const size_t kc = static_cast<size_t>(std::min<int64_t>(cap_cells, *ncells));
     if (kp) std::memcpy(patches, l.patches.data(), kp * sizeof(PatchDesc));
     if (kc) std::memcpy(cells, l.cells.data(), kc * sizeof(PatchCell));
+    return COSTA_OK;
+}
+
+costa_status costa_debug_dispatch(int n, const costa_layout *A, const costa_layout *B, const costa_op *ops,
+                                  int64_t *out) {
+    if (n < 1 || n > 65535 || !A || !B || !ops || !out) return fail(COSTA_ERR_INVALID_ARG, "bad arguments");
+    Plan plan;
+    for (int k = 0; k < n; ++k) {
+        costa_status s = validate_pair(A[k], B[k], ops[k]);
+        if (s != COSTA_OK) return s;
+        if (A[k]->dt != A[0]->dt) return fail(COSTA_ERR_DTYPE, "batch mixes element types");
+    }
+    plan.dtype = A[0]->dt;
+    plan.esize = esize_of(plan.dtype);
+    plan.ts = tile_extent(plan.esize);
+    for (int k = 0; k < n; ++k) plan.probs.push_back(make_problem(A[k], B[k], ops[k], plan.ts));
+    DirectLists l;
+    const costa_status s = direct_lists(plan, l);
+    if (s != COSTA_OK) return s;
+    const int64_t v[10] = {l.patch_kinds, static_cast<int64_t>(l.patches.patches.size()),
+                           static_cast<int64_t>(l.patches.cells.size()), l.rest ? 1 : 0,
+                           static_cast<int64_t>(l.split.big.size()), static_cast<int64_t>(l.split.mis.size()),
+                           static_cast<int64_t>(l.split.pieces.size()), static_cast<int64_t>(l.halves.size()),
+                           l.tma_big, l.tma_halves};
+    std::memcpy(out, v, sizeof v);
     return COSTA_OK;
 }
 

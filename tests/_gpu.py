@@ -11,6 +11,19 @@ from workloads.materialize import DeviceMatrix, HostMatrix, host_problem
 SENTINEL = {"f32": -77.25, "f64": -77.25, "c64": complex(-77.25, 3.5), "c128": complex(-77.25, 3.5)}
 
 
+def kind_name(dtype, alpha, beta) -> str:
+    """The combine kind of a problem's scalars, by its name in
+    costa_debug_dispatch."""
+    al, be = oracle.scalar(dtype, alpha), oracle.scalar(dtype, beta)
+    if al.imag or be.imag:
+        if be == 0:
+            return "cscale"
+        return "cplxr" if dtype == "c128" and al.imag == 0 else "cplx"
+    if be != 0:
+        return "axpby2" if np.frexp(abs(be.real))[0] == 0.5 else "axpby"
+    return "copy" if al == 1 else "scale"
+
+
 class OnDevice:
     def __init__(self, prob, device, guard: int = 0, B_host=None, A_host=None):
         import paper_2106_06601_gb300 as costa
@@ -36,6 +49,15 @@ class OnDevice:
                                       relabel=relabel, stream=stream, mode=mode)
         torch.cuda.synchronize(self.device)
         return sigma
+
+    def lists(self) -> set:
+        """The work lists that a direct call of this problem runs (the planner's
+        own choice)."""
+        import paper_2106_06601_gb300 as costa
+        d = costa.costa_debug_dispatch([self.LA], [self.LB], [self.p.op])
+        patches = kind_name(self.p.dtype, self.p.alpha, self.p.beta) in d["patch_kinds"]
+        tiles = {k for k in ("tiles", "misaligned", "pieces") if d[k]}
+        return ({"patches"} if patches else set()) | (tiles if d["tiles_are_rest"] or not patches else set())
 
     def reset_A(self):
         self.Ad.upload(self.Ah)

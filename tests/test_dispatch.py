@@ -1,0 +1,146 @@
+"""The planner's choice of work lists (costa_debug_dispatch), on the CPU: for
+each line of the rule the kinds that run on patches on both of its sides, and
+that every kind has a list that covers it."""
+import numpy as np
+import pytest
+
+from workloads import layouts as L
+
+costa = pytest.importorskip("paper_2106_06601_gb300")
+
+FAKE = 1 << 40
+ES = {"f32": 4, "f64": 8, "c64": 8, "c128": 16}
+REAL = {"copy", "scale", "axpby", "axpby2"}
+OF = {"f32": REAL, "f64": REAL, "c64": REAL | {"cplx", "cscale"}, "c128": REAL | {"cplx", "cscale", "cplxr"}}
+
+
+def _layout(spec, dtype):
+    ptrs = FAKE + spec.buf.astype(np.int64) * (1 << 34) + spec.off * ES[dtype]
+    return costa.costa_layout_from_spec(spec, dtype, ptrs)
+
+
+def _pair(dtype, op, mb, ma, m, n, pads=(0, 0), grid=2):
+    B = L.block_cyclic(*((m, n) if op == "N" else (n, m)), mb, mb, grid, grid, ld_pad=pads[0], name="B")
+    A = L.block_cyclic(m, n, ma, ma, grid, grid, grid_order="C", ld_pad=pads[1], name="A")
+    return A, B
+
+
+def dispatch(dtype, *problems):
+    """costa_debug_dispatch of (A, B, op) specs, the kinds those of the type."""
+    As, Bs = [_layout(A, dtype) for A, _, _ in problems], [_layout(B, dtype) for _, B, _ in problems]
+    try:
+        d = costa.costa_debug_dispatch(As, Bs, [op for _, _, op in problems])
+    finally:
+        for x in As + Bs:
+            x.destroy()
+    for key in ("patch_kinds", "tma_kinds", "tma_halves_kinds"):
+        d[key] &= OF[dtype]
+    # every kind has a list: patches, or tiles that are not only other problems'
+    assert d["patches"] > 0 if d["patch_kinds"] else d["patches"] == 0
+    tiles = d["tiles"] + d["misaligned"] + d["pieces"]
+    assert tiles > 0 or d["patch_kinds"] == OF[dtype] or all(A.numel() == 0 for A, _, _ in problems)
+    if not d["tiles_are_rest"]:
+        assert d["patch_kinds"] and tiles > 0
+    return d
+
+
+def kinds(dtype, op, mb, ma, m, n=None, pads=(0, 0), grid=2):
+    A, B = _pair(dtype, op, mb, ma, m, n or m, pads, grid)
+    return dispatch(dtype, (A, B, op))["patch_kinds"]
+
+
+ALL, NONE = REAL, set()
+
+
+@pytest.mark.parametrize("dtype, op, mb, ma, m, n, pads, want", [
+    # small, partial or misaligned tiles, whatever the size
+    ("f64", "T", 50, 75, 150, 171, (0, 0), ALL),
+    ("f64", "T", 24, 100, 1200, 1200, (0, 0), ALL),
+    ("f32", "T", 24, 100, 1200, 1200, (0, 0), NONE),  # 4-byte partial tiles stay
+    ("f64", "T", 64, 128, 2048, 2048, (1, 0), ALL),
+    ("f32", "T", 64, 128, 2048, 2048, (0, 1), ALL),
+    ("f32", "T", 64, 128, 2048, 2048, (1, 0), NONE),  # only the source misaligned: windows
+    ("f64", "T", 64, 64, 7001, 6003, (0, 0), ALL),    # a twentieth misaligned
+    # in large lists, tiles along A's runs from 16 x 16 on are not poor
+    ("f64", "N", 24, 24, 1200, 1200, (0, 0), ALL),
+    ("f64", "N", 24, 24, 3072, 3072, (0, 0), NONE),
+    # power-of-two cells of doubles keep the kinds that read A on tiles in lists of middle size
+    ("f64", "T", 8, 8, 1544, 1544, (0, 0), ALL),
+    ("f64", "T", 8, 8, 1552, 1552, (0, 0), {"copy", "scale"}),
+    ("f64", "T", 8, 8, 4464, 4464, (0, 0), {"copy", "scale"}),
+    ("f64", "T", 8, 8, 4480, 4480, (0, 0), {"copy", "scale", "axpby2"}),
+    ("f64", "T", 8, 8, 7064, 7064, (0, 0), {"copy", "scale", "axpby2"}),
+    ("f64", "T", 8, 8, 7072, 7072, (0, 0), ALL),
+    ("c64", "T", 8, 8, 2048, 2048, (0, 0), OF["c64"]),
+    # ... a lower line where lines of B are shared
+    ("f64", "N", 64, 8, 2816, 2816, (0, 0), {"copy", "scale"}),
+    ("f64", "N", 64, 8, 2832, 2832, (0, 0), ALL),
+    # ... and alpha b with blocks of different sizes
+    ("f64", "T", 8, 64, 3136, 3136, (0, 0), {"copy", "scale"}),
+    ("f64", "T", 8, 64, 3200, 3200, (0, 0), {"copy"}),
+    ("f64", "T", 64, 8, 4416, 4416, (0, 0), {"copy"}),
+    ("f64", "T", 64, 8, 4480, 4480, (0, 0), {"copy", "scale", "axpby2"}),
+    # 8-byte copies of partial tiles stay up to 1.75 times the L2
+    ("f64", "T", 48, 48, 2832, 2832, (0, 0), {"scale"}),
+    ("f64", "T", 48, 48, 3840, 3840, (0, 0), {"copy", "scale"}),
+    # f32 cells of 16 x 16 and more, block ratio no power of two
+    ("f32", "T", 16, 48, 8064, 8064, (0, 0), {"axpby", "axpby2"}),
+    ("f32", "T", 48, 16, 8064, 8064, (0, 0), NONE),
+    ("f32", "T", 16, 32, 8064, 8064, (0, 0), ALL),
+])
+def test_lists_of_poor_tiles(dtype, op, mb, ma, m, n, pads, want):
+    assert kinds(dtype, op, mb, ma, m, n, pads) == want
+
+
+@pytest.mark.parametrize("dtype, op, mb, ma, m, want", [
+    ("f64", "T", 64, 128, 3712, NONE),  # 1.75 times the L2
+    ("f64", "T", 64, 128, 3840, {"copy", "axpby2"}),
+    ("f64", "N", 64, 128, 3840, {"copy", "axpby2"}),
+    ("c64", "T", 64, 128, 3840, OF["c64"]),
+    ("c128", "T", 64, 128, 6016, NONE),
+    ("f32", "T", 64, 128, 5632, NONE),  # twice the L2
+    ("f32", "T", 64, 128, 5760, ALL),
+    ("f64", "T", 40, 40, 8000, {"copy", "axpby", "axpby2"}),  # TMA could stage too few tiles
+    ("f32", "T", 24, 100, 8000, NONE),  # ragged cells
+    ("f32", "T", 48, 96, 8064, {"axpby", "axpby2"}),  # cells meet inside most patches
+    ("f32", "N", 48, 96, 8064, ALL),
+    ("f32", "T", 96, 48, 6144, NONE),  # ... A's blocks the smaller ones
+    ("f32", "T", 96, 48, 7104, {"axpby", "axpby2"}),
+])
+def test_lists_of_full_tiles(dtype, op, mb, ma, m, want):
+    assert kinds(dtype, op, mb, ma, m) == want
+
+
+def test_targets_of_whole_runs_stay_on_tiles():
+    """16-row panels: every target tile is one contiguous run."""
+    m, n = 16384, 4096
+    A = L.block_cyclic(m, n, 16, n, m // 16, 1, name="A")
+    B = L.block_cyclic(n, m, 64, 64, m // 16, 1, name="B")
+    assert dispatch("f64", (A, B, "T"))["patch_kinds"] == NONE
+
+
+def test_mixed_element_orders_stay_on_tiles():
+    """Layouts that mix element orders have no patches; in a batch the other
+    problems move to patches, and every kind runs on both lists."""
+    B = L.block_cyclic(70, 90, 5, 7, 2, 2, name="B")
+    order = np.zeros((2, 3), np.int32)
+    order[0, 1] = 1
+    mixed = L.packed_blocks([0, 33, 90], [0, 20, 41, 70], np.arange(6).reshape(2, 3) % 4, 4, order=order)
+    plain = L.block_cyclic(90, 70, 3, 11, 2, 2, name="A")
+    d = dispatch("f64", (mixed, B, "T"))
+    assert d["patch_kinds"] == NONE and d["tiles"] + d["misaligned"] + d["pieces"] > 0
+    d = dispatch("f64", (plain, B, "T"))
+    assert d["patch_kinds"] == ALL and d["tiles"] + d["misaligned"] + d["pieces"] == 0
+    d = dispatch("f64", (mixed, B, "T"), (plain, B, "T"))
+    assert d["patch_kinds"] == ALL and d["tiles_are_rest"] and d["tiles"] + d["misaligned"] + d["pieces"] > 0
+
+
+@pytest.mark.parametrize("dtype", ["f64", "c128", "f32"])
+def test_empty_problems_in_a_batch(dtype):
+    """A problem without elements neither has patches nor keeps the others from
+    theirs."""
+    A, B = _pair(dtype, "T", 5, 7, 70, 90)
+    empty = L.packed_blocks([0], [0, 5], np.zeros((0, 1), np.int32), 4)
+    empty_b = L.packed_blocks([0, 5], [0], np.zeros((1, 0), np.int32), 4)
+    assert dispatch(dtype, (empty, empty_b, "T"), (A, B, "T"))["patch_kinds"] == OF[dtype]
+    assert dispatch(dtype, (empty, empty_b, "T"))["patch_kinds"] == NONE

@@ -26,9 +26,12 @@ def dev():
     return d
 
 
-def check_problem(p, dev, mode="direct", relabel=True, guard=0):
+def check_problem(p, dev, mode="direct", relabel=True, guard=0, lists=None):
+    """Runs p and compares it with the oracle; `lists`: the work lists that a
+    direct call must run (None: any)."""
     g = OnDevice(p, dev, guard=guard)
     try:
+        assert lists is None or g.lists() == lists
         sigma = g.run(relabel=relabel, mode=mode)
         got = g.Ad.download()
         want = g.oracle_result()
@@ -47,8 +50,8 @@ def test_fuzz_direct(case, dev):
 
 @pytest.mark.parametrize("case", range(96))
 def test_small_blocks(case, dev):
-    """Small and odd blocks: the small-tile kernel's pieces and groups, in
-    direct and message mode (the two agree bit for bit)."""
+    """Small and odd blocks: patches in direct mode, the small-tile kernel's
+    pieces and groups in message mode (the two agree bit for bit)."""
     p = C.small_block_problem(case)
     _, direct = check_problem(p, dev)
     _, msg = check_problem(p, dev, mode="message")
@@ -341,9 +344,12 @@ def test_transform_replays_in_cuda_graph(dev):
 @pytest.mark.parametrize("op", ["N", "T", "C"])
 def test_misaligned_runs(dtype, op, dev):
     """Runs off 16-byte boundaries: odd leading dimensions, odd block sizes
-    and buffers at odd element offsets (guards).  Copy and scale take the
-    16-byte window path, the kinds that read A the element path; both must
-    write every element of A once and nothing outside A's blocks."""
+    and buffers at odd element offsets (guards).  Direct calls run on patches;
+    the lists of message mode, and direct ones of layouts that mix element
+    orders, on the misaligned instance of the tile kernel: copy and scale take
+    its 16-byte window path (f32: with aligned target runs), the kinds that read
+    A its element path.  All must write every element of A once and nothing
+    outside A's blocks."""
     m, n = 150, 171
     am, an = (m, n) if op == "N" else (n, m)
     for k, (pad_b, pad_a, guard) in enumerate(((1, 0, 0), (0, 3, 0), (2, 1, 3), (3, 2, 1))):
@@ -352,12 +358,22 @@ def test_misaligned_runs(dtype, op, dev):
         for alpha, beta in ((1.0, 0.0), (2.0, 0.0), (2.0, 0.5), (-0.3, 0.7)):
             p = C.Problem("misaligned", dtype, op, alpha, beta, A, B, "uniform",
                           "nan" if beta == 0 else "uniform", C.SEED0 + 11 + k)
-            check_problem(p, dev, guard=guard)
+            _, direct = check_problem(p, dev, guard=guard, lists={"patches"})
+            _, msg = check_problem(p, dev, mode="message", guard=guard)
+            assert np.array_equal(msg.arena, direct.arena, equal_nan=True)
+            order = np.zeros((5, 7), np.int32)
+            order[1 + k % 3, 2 + k] = 1  # one block in the other order: no patches
+            A2 = L.packed_blocks(np.linspace(0, am, 6).astype(int), np.linspace(0, an, 8).astype(int),
+                                 np.arange(35).reshape(5, 7) % 6, 6, order=order, ld_pad=pad_a)
+            p2 = C.Problem("mixed", dtype, op, alpha, beta, A2, B, "uniform",
+                           "nan" if beta == 0 else "uniform", C.SEED0 + 11 + k)
+            check_problem(p2, dev, guard=guard, lists={"misaligned"})
 
 
 def _complex_layouts(op):
     """Aligned multi-tile grid with a ragged tail, odd leading dimensions
-    (misaligned runs) and 8 x 8 blocks (the small-tile kernel)."""
+    (misaligned runs) and 8 x 8 blocks; the last two run on patches in direct
+    mode and on the misaligned and small-tile kernels in message mode."""
     m, n = 150, 171
     am, an = (m, n) if op == "N" else (n, m)
     yield L.block_cyclic(m, n, 40, 24, 2, 3), L.block_cyclic(am, an, 33, 64, 3, 2, grid_order="C")
@@ -396,6 +412,9 @@ def test_complex_scalars_within_2ulp(dtype, op, alpha, beta, dev):
             got, want = g.Ad.download(), g.oracle_result()
             compare(p, got, want, g.Ah, g.Bh)
             assert np.array_equal(g.Bd.download().arena, g.Bh.arena, equal_nan=True)
+            g.reset_A()
+            g.run(mode="message")
+            assert np.array_equal(g.Ad.download().arena, got.arena, equal_nan=True)
             if beta == 0:
                 assert not np.isnan(global_matrix(p.A, got.buffers())).any()
             al, be = oracle.scalar(dtype, alpha), oracle.scalar(dtype, beta)
