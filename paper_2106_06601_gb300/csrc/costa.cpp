@@ -635,10 +635,12 @@ costa_status direct_lists(const Plan &plan, DirectLists &out) {
     out.had_halves = !out.halves.empty();
     out.split.big = cut_few(std::move(out.split.big), es);
     out.halves = cut_few(std::move(out.halves), es);
-    // TMA staging (tma.cpp): the kinds the policy would give it; their lists
-    // are built by the first call of such a kind (ensure_tma)
-    out.tma_big = tma_policy_kinds(out.split.big, es, cplx, false);
-    out.tma_halves = out.had_halves ? tma_policy_kinds(out.halves, es, cplx, true) : 0;
+    // TMA staging (tma.cpp): the kinds the policy would give it, of those that
+    // run on these tiles; their lists are built by the first call of such a
+    // kind (ensure_tma)
+    const uint32_t on_tiles = out.rest ? kAllKinds : kAllKinds & ~out.patch_kinds;
+    out.tma_big = tma_policy_kinds(out.split.big, es, cplx, false) & on_tiles;
+    out.tma_halves = out.had_halves ? tma_policy_kinds(out.halves, es, cplx, true) & on_tiles : 0;
     return COSTA_OK;
 }
 

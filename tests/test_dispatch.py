@@ -41,6 +41,8 @@ def dispatch(dtype, *problems):
     assert tiles > 0 or d["patch_kinds"] == OF[dtype] or all(A.numel() == 0 for A, _, _ in problems)
     if not d["tiles_are_rest"]:
         assert d["patch_kinds"] and tiles > 0
+        # no TMA lists for kinds that do not run on these tiles
+        assert not (d["tma_kinds"] | d["tma_halves_kinds"]) & d["patch_kinds"]
     return d
 
 
@@ -109,6 +111,15 @@ def test_lists_of_poor_tiles(dtype, op, mb, ma, m, n, pads, want):
 ])
 def test_lists_of_full_tiles(dtype, op, mb, ma, m, want):
     assert kinds(dtype, op, mb, ma, m) == want
+
+
+def test_tma_lists_only_for_kinds_on_tiles():
+    """The general beta of doubles is staged by TMA where it runs on tiles, and
+    has no TMA lists to build on its first call where it runs on patches."""
+    for mb, m, want in ((64, 3840, {"axpby"}), (40, 8000, set())):
+        A, B = _pair("f64", "T", mb, 2 * mb if mb == 64 else mb, m, m)
+        d = dispatch("f64", (A, B, "T"))
+        assert not d["tiles_are_rest"] and d["tma_kinds"] == want and not d["tma_halves_kinds"]
 
 
 def test_targets_of_whole_runs_stay_on_tiles():
