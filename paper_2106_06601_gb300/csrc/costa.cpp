@@ -454,7 +454,7 @@ bool uneven(const ProblemHost &ph) {
 
 uint32_t take_patches(const Plan &plan, std::vector<TileDesc> &list, PatchList &out, bool &rest) {
     rest = true;
-    if (list.empty()) return 0;
+    if (list.empty() || tma_mode() == 1) return 0;  // COSTA_TMA=1: every kind through the TMA tiles
     const int es = plan.esize;
     const bool cplx = plan.dtype == COSTA_C64 || plan.dtype == COSTA_C128;
     int64_t all = 0;
@@ -551,7 +551,7 @@ uint32_t take_patches(const Plan &plan, std::vector<TileDesc> &list, PatchList &
         return kAllKinds;
     }
     if (es == 16 || !beyond || 2 * runs >= all || 2 * small >= all ||
-        2 * src_mis >= all || (es == 4 && 2 * part >= all) || tma_mode() == 1)
+        2 * src_mis >= all || (es == 4 && 2 * part >= all))
         return 0;
     if (es == 4)  // transposed sources whose columns lie a multiple of 32 KB apart
         for (const ProblemHost &ph : plan.probs)
@@ -633,8 +633,10 @@ costa_status direct_lists(const Plan &plan, DirectLists &out) {
     for (int k = 0; k < n; ++k) halve[k] = any && use_halves(plan.probs[k], es);
     out.halves = split_x_halves(out.split.big, ts / 2, es, halve);
     out.had_halves = !out.halves.empty();
-    out.split.big = cut_few(std::move(out.split.big), es);
-    out.halves = cut_few(std::move(out.halves), es);
+    if (tma_mode() != 1) {  // (COSTA_TMA=1: a TMA tile is 16 or 32 runs of whole 128-byte boxes)
+        out.split.big = cut_few(std::move(out.split.big), es);
+        out.halves = cut_few(std::move(out.halves), es);
+    }
     // TMA staging (tma.cpp): the kinds the policy would give it, of those that
     // run on these tiles; their lists are built by the first call of such a
     // kind (ensure_tma)

@@ -1,6 +1,10 @@
 """The planner's choice of work lists (costa_debug_dispatch), on the CPU: for
 each line of the rule the kinds that run on patches on both of its sides, and
 that every kind has a list that covers it."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -8,6 +12,7 @@ from workloads import layouts as L
 
 costa = pytest.importorskip("paper_2106_06601_gb300")
 
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 FAKE = 1 << 40
 ES = {"f32": 4, "f64": 8, "c64": 8, "c128": 16}
 REAL = {"copy", "scale", "axpby", "axpby2"}
@@ -120,6 +125,23 @@ def test_tma_lists_only_for_kinds_on_tiles():
         A, B = _pair("f64", "T", mb, 2 * mb if mb == 64 else mb, m, m)
         d = dispatch("f64", (A, B, "T"))
         assert not d["tiles_are_rest"] and d["tma_kinds"] == want and not d["tma_halves_kinds"]
+
+
+def test_tma_for_every_kind_keeps_patches_off():
+    """COSTA_TMA=1 (read once per process) stages every kind's tiles by TMA, so
+    nothing runs on patches."""
+    script = """
+from tests.test_dispatch import REAL, _pair, dispatch
+for args in (("f64", "T", 40, 40, 600, 640), ("f64", "T", 24, 100, 1200, 1200), ("f64", "T", 64, 128, 3840, 3840),
+             ("c128", "N", 8, 8, 300, 300), ("f32", "T", 50, 75, 300, 300)):
+    A, B = _pair(*args)
+    d = dispatch(args[0], (A, B, args[1]))
+    assert not d["patch_kinds"], args
+    assert not d["tiles"] or d["tma_kinds"] >= REAL, args
+"""
+    r = subprocess.run([sys.executable, "-c", script], cwd=ROOT, env=dict(os.environ, COSTA_TMA="1"),
+                       capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-3000:]
 
 
 def test_targets_of_whole_runs_stay_on_tiles():

@@ -1,7 +1,8 @@
 """TMA staging of the tile kernel's source tiles (COSTA_TMA=1, read when a
-plan is built): in a fresh process with the variable set, the configurations
-and fuzz problems take the TMA instance of the tile kernel and must give the
-oracle's result (bit for bit in the exact class, else within the tolerance),
+plan is built): in a fresh process with the variable set, the configurations,
+one pair of aligned layouts in every type, op and kind, and the few fuzz
+problems with tiles that qualify take the TMA instance of the tile kernel and
+must give the oracle's result (bit for bit in the exact class, else within the tolerance),
 with no TMA wait giving up."""
 import os
 import subprocess
@@ -35,6 +36,25 @@ for case in range(int(sys.argv[1])):
     assert st["timeouts"] == 0, st
     used += st["tiles"] + st["halves_tiles"]
     g.close()
+if int(sys.argv[1]):  # every type, op and kind on tiles that TMA stages
+    from workloads import layouts as L
+    for dtype in ("f32", "f64", "c64", "c128"):
+        for op in "NTC":
+            # f32 tiles are halved unless A's blocks are longer than 256; halves of
+            # op = N have runs of 64 bytes, which TMA does not take
+            B = L.block_cyclic(*((320, 192) if op == "N" else (192, 320)), 64, 64, 2, 2)
+            A = L.block_cyclic(320, 192, 512 if dtype == "f32" else 128, 32, 2, 2, grid_order="C")
+            cases = [(1.0, 0.0), (-0.7, 0.0), (-0.3, 0.7), (2.0, -0.5)]
+            if dtype[0] == "c":
+                cases += [(0.3 - 0.4j, 0.0), (-1.5, 0.3 + 0.7j), (1 + 0.5j, 0.5 - 0.25j)]
+            for alpha, beta in cases:
+                p = C.Problem("tma", dtype, op, alpha, beta, A, B, "uniform", "nan" if beta == 0 else "uniform", C.SEED0 + 18)
+                g = OnDevice(p, dev)
+                g.run()
+                compare(p, g.Ad.download(), g.oracle_result(), g.Ah, g.Bh)
+                st = costa.costa_debug_tma(g.LA, g.LB, p.op)
+                assert st["timeouts"] == 0 and st["tiles"] > 0 and st["kinds"] > 0, (dtype, op, st)
+                g.close()
 for name in sys.argv[2:]:
     p = C.CONFIGS[name]() if name in C.CONFIGS else C.c2()
     if name == "c2beta":  # c2's layouts with a general beta: the kind TMA serves by default
