@@ -439,8 +439,16 @@ constexpr uint32_t kAllKinds = (1u << K_NKINDS) - 1u;
 constexpr uint32_t kAlignedPatchKinds = (1u << K_COPY) | (1u << K_AXPBY2);  // f64; f32, c64: all
 constexpr int64_t kL2Bytes = int64_t(126) << 20;
 
-// Whether the larger of A's and op(B)'s (first) blocks is, along some axis,
-// no power of two times the smaller one.
+// The longest block along one axis (a submatrix starts and ends with parts of
+// blocks).
+int64_t block_extent(const std::vector<int64_t> &splits) {
+    int64_t e = 0;
+    for (size_t k = 1; k < splits.size(); ++k) e = std::max(e, splits[k] - splits[k - 1]);
+    return e;
+}
+
+// Whether the larger of A's and op(B)'s blocks is, along some axis, no power
+// of two times the smaller one.
 bool uneven(const ProblemHost &ph) {
     const costa_layout_s &A = *ph.A, &B = *ph.B;
     const bool t = ph.op != COSTA_OP_N;
@@ -448,8 +456,7 @@ bool uneven(const ProblemHost &ph) {
         const int64_t lo = std::max<int64_t>(std::min(a, b), 1), q = std::max(a, b) / lo;
         return lo * q != std::max(a, b) || (q & (q - 1)) != 0;
     };
-    return odd(A.R[1] - A.R[0], t ? B.C[1] - B.C[0] : B.R[1] - B.R[0]) ||
-           odd(A.C[1] - A.C[0], t ? B.R[1] - B.R[0] : B.C[1] - B.C[0]);
+    return odd(block_extent(A.R), block_extent(t ? B.C : B.R)) || odd(block_extent(A.C), block_extent(t ? B.R : B.C));
 }
 
 uint32_t take_patches(const Plan &plan, std::vector<TileDesc> &list, PatchList &out, bool &rest) {

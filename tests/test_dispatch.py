@@ -118,6 +118,21 @@ def test_lists_of_full_tiles(dtype, op, mb, ma, m, want):
     assert kinds(dtype, op, mb, ma, m) == want
 
 
+@pytest.mark.parametrize("mb, ma, off, want", [(16, 32, 4, ALL), (16, 32, 0, ALL), (16, 48, 16, {"axpby", "axpby2"}),
+                                               (16, 48, 32, {"axpby", "axpby2"})])
+def test_block_sizes_of_submatrices(mb, ma, off, want):
+    """A submatrix starts with a part of a block: the rule compares the block
+    sizes, not these parts (12 against 28 for BC16 -> BC32 from element 4 on, 16
+    against 32 or 16 for BC16 -> BC48 from 16 or 32 on)."""
+    n = 8064
+    full = off + n
+    lld = [f[2] for f in L.scalapack_full(full, full, ma, ma, 0, 0, 2, 2, "C", ld_pad=0)]
+    A = L.scalapack_sub(full, full, ma, ma, 0, 0, 2, 2, "C", off + 1, off + 1, n, n, [v + -v % 4 for v in lld])
+    lld = [f[2] for f in L.scalapack_full(full, full, mb, mb, 0, 0, 2, 2, "R", ld_pad=0)]
+    B = L.scalapack_sub(full, full, mb, mb, 0, 0, 2, 2, "R", off + 1, off + 1, n, n, [v + -v % 4 for v in lld])
+    assert dispatch("f32", (A, B, "T"))["patch_kinds"] == want
+
+
 def test_tma_lists_only_for_kinds_on_tiles():
     """The general beta of doubles is staged by TMA where it runs on tiles, and
     has no TMA lists to build on its first call where it runs on patches."""
