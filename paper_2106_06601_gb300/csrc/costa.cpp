@@ -425,10 +425,12 @@ costa_status check_access(costa_layout_s *L, int dev, const char *which) {
 // of 16-row panels (one run per tile) 1900 -> 1885 with three times the list.
 // f32 T copy 87 -> 84, T beta = 0.7 135 -> 130, N beta = 0.5 130 -> 127, 64
 // matrices of 2048 x 3072 515 -> 489, 7001 x 6003 T copy 64 -> 56, N beta = 0.5
-// 94 -> 85; but 4096^2 T copy 23.8 -> 24.6, and one 8192^2 matrix (columns 32 KB
-// apart) T 89 -> 95, and cells below three quarters of a patch whose extents
-// are no multiples of 16 (BC24 -> BC100) T copy 110 -> 127: these stay.  f32
-// copies stay where transposed patches take more than 1.25 cells on average
+// 94 -> 85; but 4096^2 T copy 23.8 -> 24.6, and cells below three quarters of a
+// patch whose extents are no multiples of 16 (BC24 -> BC100) T copy 110 -> 127:
+// these stay.  f32 copies stay where at least half of the list is transposed from
+// columns that lie a multiple of 32 KB apart (one 8192^2 matrix T copy 87 -> 92,
+// beta = 0.5 134 -> 128, N copy 86.7 -> 86.1; 16384 x 8192 174 -> 181, 265 -> 248),
+// and where transposed patches take more than 1.25 cells on average
 // (BC48 -> BC96 copy 88 -> 101, beta = 0.5 133 -> 132; BC56 -> BC112 89 -> 107,
 // 142 -> 135), and every kind if A's blocks are the smaller ones, below 7000^2
 // (BC96 -> BC32 6144^2 beta = 0.5 74 -> 75).  c128 copy (16384^2) 1321 -> 1329 stays on the tiles.
@@ -436,6 +438,7 @@ costa_status check_access(costa_layout_s *L, int dev, const char *which) {
 // `rest`: the tiles left in `list` are other problems' than the patches'
 // (reason 1), not the same problems' for the other kinds.
 constexpr uint32_t kAllKinds = (1u << K_NKINDS) - 1u;
+constexpr uint32_t kCopies = (1u << K_COPY) | (1u << K_SCALE);
 constexpr uint32_t kAlignedPatchKinds = (1u << K_COPY) | (1u << K_AXPBY2);  // f64; f32, c64: all
 constexpr int64_t kL2Bytes = int64_t(126) << 20;
 
@@ -475,7 +478,7 @@ uint32_t take_patches(const Plan &plan, std::vector<TileDesc> &list, PatchList &
     const bool many = all >= 3000000;
     struct Sums {  // elements by what their tiles are
         int64_t poor = 0, mis = 0, runs = 0, boxes = 0, small = 0, src_mis = 0, part = 0, neat = 0, coarse = 0, fine = 0,
-                trans = 0, odd16 = 0;
+                trans = 0, odd16 = 0, wide = 0;
     };
     auto count = [&](const TileDesc &d, Sums &c) {
         const int64_t e = static_cast<int64_t>(d.nx) * d.ny;
@@ -498,6 +501,7 @@ uint32_t take_patches(const Plan &plan, std::vector<TileDesc> &list, PatchList &
         if (r & 1) c.coarse += e;
         if (r & 2) c.fine += e;
         if (tr) c.trans += e;
+        if (tr && static_cast<int64_t>(d.sld) * es % 32768 == 0) c.wide += e;
         if ((r & 4) && tr && (d.flags & TF_FAST) && d.nx >= 16 && d.ny >= 16) c.odd16 += e;
         if (run) c.runs += e;
         const int nr = tr ? d.nx : d.ny, len = tr ? d.ny : d.nx;
@@ -514,10 +518,11 @@ uint32_t take_patches(const Plan &plan, std::vector<TileDesc> &list, PatchList &
         }
     });
     int64_t poor = 0, mis = 0, runs = 0, boxes = 0, small = 0, src_mis = 0, part = 0, neat = 0, coarse = 0, fine = 0,
-            trans = 0, odd16 = 0;
+            trans = 0, odd16 = 0, wide = 0;
     for (const Sums &c : part_sums) {
         poor += c.poor, mis += c.mis, runs += c.runs, boxes += c.boxes, small += c.small, src_mis += c.src_mis;
         part += c.part, neat += c.neat, coarse += c.coarse, fine += c.fine, trans += c.trans, odd16 += c.odd16;
+        wide += c.wide;
     }
     const size_t n = plan.probs.size();
     const bool beyond = 8 * all * es > (es == 8 ? 7 : 8) * kL2Bytes;  // B and A: 1.75 or 2 times the L2
@@ -541,7 +546,7 @@ uint32_t take_patches(const Plan &plan, std::vector<TileDesc> &list, PatchList &
         }
         if (es == 4 && mis == 0 && 4 * odd16 >= 3 * all && all >= 2400000 &&
             std::find(taken.begin(), taken.end(), 0) == taken.end())
-            stay = 2 * coarse >= all ? kAllKinds : (1u << K_COPY) | (1u << K_SCALE);
+            stay = 2 * coarse >= all ? kAllKinds : kCopies;
         if (stay == kAllKinds) {
             out.patches.clear();
             out.cells.clear();
@@ -560,9 +565,6 @@ uint32_t take_patches(const Plan &plan, std::vector<TileDesc> &list, PatchList &
     if (es == 16 || !beyond || 2 * runs >= all || 2 * small >= all ||
         2 * src_mis >= all || (es == 4 && 2 * part >= all))
         return 0;
-    if (es == 4)  // transposed sources whose columns lie a multiple of 32 KB apart
-        for (const ProblemHost &ph : plan.probs)
-            if (!ph.B->blocks.empty() && static_cast<int64_t>(ph.B->blocks[0].ld) * es % 32768 == 0) return 0;
     for (size_t k = 0; k < n; ++k)
         if (!append_patches(plan.probs[k], static_cast<int>(k), all, out)) {
             out.patches.clear();
@@ -575,12 +577,13 @@ uint32_t take_patches(const Plan &plan, std::vector<TileDesc> &list, PatchList &
         out.cells.clear();
         return 0;
     }
-    if (!cut && (es == 4 || cplx || mis > 0)) {
+    const bool copies_stay = cut || (es == 4 && 2 * wide >= all);
+    if (!copies_stay && (es == 4 || cplx || mis > 0)) {
         list.clear();
         return kAllKinds;
     }
     rest = false;
-    if (cut) return kAllKinds & ~((1u << K_COPY) | (1u << K_SCALE));
+    if (copies_stay) return kAllKinds & ~kCopies;
     return kAlignedPatchKinds | (4 * boxes < 3 * all ? 1u << K_AXPBY : 0u);
 }
 

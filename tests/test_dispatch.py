@@ -159,6 +159,26 @@ for args in (("f64", "T", 40, 40, 600, 640), ("f64", "T", 24, 100, 1200, 1200), 
     assert r.returncode == 0, r.stderr[-3000:]
 
 
+@pytest.mark.parametrize("op, m, n, grid, want", [
+    ("T", 8192, 8192, 1, {"axpby", "axpby2"}), ("N", 8192, 8192, 1, ALL), ("T", 8192, 8192, 2, ALL),
+    ("T", 16384, 16384, 2, {"axpby", "axpby2"}), ("N", 16384, 16384, 2, ALL), ("T", 8192, 8064, 1, ALL)])
+def test_f32_columns_a_multiple_of_32_kb_apart(op, m, n, grid, want):
+    """Only transposed copies stay on tiles for it (the leading dimension of a
+    rank's source is its rows: n / grid transposed, m / grid otherwise)."""
+    assert kinds("f32", op, 64, 128, m, n, (0, 0), grid) == want
+
+
+def test_f32_columns_32_kb_apart_count_by_their_share():
+    """One problem of a batch, or an empty first block, does not decide for the
+    whole list."""
+    wide, plain = _pair("f32", "T", 64, 128, 8192, 8192, grid=1), _pair("f32", "T", 64, 128, 8192, 8064, grid=1)
+    assert dispatch("f32", (*wide, "T"), (*plain, "T"), (*plain, "T"))["patch_kinds"] == ALL
+    assert dispatch("f32", (*plain, "T"), (*wide, "T"), (*wide, "T"))["patch_kinds"] == {"axpby", "axpby2"}
+    A = L.packed_blocks(np.arange(0, 8193, 128), np.arange(0, 8193, 128), np.zeros((64, 64)), 1)
+    B = L.packed_blocks([0, 0, 8192], [0, 8192], np.zeros((2, 1)), 1)  # ld 1 of the empty block
+    assert dispatch("f32", (A, B, "T"))["patch_kinds"] == {"axpby", "axpby2"}
+
+
 def test_targets_of_whole_runs_stay_on_tiles():
     """16-row panels: every target tile is one contiguous run."""
     m, n = 16384, 4096
