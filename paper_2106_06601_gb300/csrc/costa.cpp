@@ -432,14 +432,21 @@ costa_status check_access(costa_layout_s *L, int dev, const char *which) {
 // beta = 0.5 134 -> 128, N copy 86.7 -> 86.1; 16384 x 8192 174 -> 181, 265 -> 248),
 // and where transposed patches take more than 1.25 cells on average
 // (BC48 -> BC96 copy 88 -> 101, beta = 0.5 133 -> 132; BC56 -> BC112 89 -> 107,
-// 142 -> 135), and every kind if A's blocks are the smaller ones, below 7000^2
-// (BC96 -> BC32 6144^2 beta = 0.5 74 -> 75).  c128 copy (16384^2) 1321 -> 1329 stays on the tiles.
+// 142 -> 135), and every kind if A's blocks are the smaller ones, below 7071^2
+// (BC96 -> BC48 6144^2 copy 51 -> 54, beta = 0.5 76 -> 77).  Below 6856^2 f32
+// lists of whole aligned tiles between blocks of powers of two move copies only,
+// and none along A's runs;
+// patches / tiles, four matrices in turn, BC64 -> BC128 on 4 x 4 and 2 x 2 grids,
+// BC32 -> BC64 on 4 x 4: T beta = 0.5 5760^2 1.03, 1.05, 1.03, 6592^2 1.02, 1.04,
+// 1.01, 7040^2 0.97, 1.00, 0.96; N 1.04, 1.03, 1.01, 1.03, 1.03, 0.99, 1.02, 1.02,
+// 0.96; N copy 1.02, 1.01, 1.00, 1.01, 1.01, 0.99, 1.00, 1.01, 0.98.  (BC96 -> BC96
+// 0.91 to 1.00 all over; ragged 6001 x 6003 T beta = 0.5 0.93, N copy 0.87.)  c128 copy (16384^2) 1321 -> 1329 stays on the tiles.
 // Returns the kinds that run on patches (bit per kind; 0: no patches).
 // `rest`: the tiles left in `list` are other problems' than the patches'
 // (reason 1), not the same problems' for the other kinds.
 constexpr uint32_t kAllKinds = (1u << K_NKINDS) - 1u;
 constexpr uint32_t kCopies = (1u << K_COPY) | (1u << K_SCALE);
-constexpr uint32_t kAlignedPatchKinds = (1u << K_COPY) | (1u << K_AXPBY2);  // f64; f32, c64: all
+constexpr uint32_t kAlignedPatchKinds = (1u << K_COPY) | (1u << K_AXPBY2);  // f64; c64: all
 constexpr int64_t kL2Bytes = int64_t(126) << 20;
 
 // The longest block along one axis (a submatrix starts and ends with parts of
@@ -448,6 +455,15 @@ int64_t block_extent(const std::vector<int64_t> &splits) {
     int64_t e = 0;
     for (size_t k = 1; k < splits.size(); ++k) e = std::max(e, splits[k] - splits[k - 1]);
     return e;
+}
+
+// Whether all of A's and B's block extents are powers of two.
+bool blocks_pow2(const ProblemHost &ph) {
+    for (const std::vector<int64_t> *s : {&ph.A->R, &ph.A->C, &ph.B->R, &ph.B->C}) {
+        const int64_t e = block_extent(*s);
+        if (e & (e - 1)) return false;
+    }
+    return true;
 }
 
 // Whether the larger of A's and op(B)'s blocks is, along some axis, no power
@@ -468,17 +484,18 @@ uint32_t take_patches(const Plan &plan, std::vector<TileDesc> &list, PatchList &
     const int es = plan.esize;
     const bool cplx = plan.dtype == COSTA_C64 || plan.dtype == COSTA_C128;
     int64_t all = 0;
-    std::vector<char> ratio;  // per problem: 1 B's blocks the larger ones, 2 A's, 4 uneven
+    std::vector<char> ratio;  // per problem: 1 B's blocks the larger ones, 2 A's, 4 uneven, 8 powers of two
     ratio.reserve(plan.probs.size());
     for (const ProblemHost &ph : plan.probs) {
         all += ph.A->m * ph.A->n;
         const int64_t na = int64_t(ph.A->nbr) * ph.A->nbc, nb = int64_t(ph.B->nbr) * ph.B->nbc;
-        ratio.push_back(static_cast<char>((2 * nb <= na ? 1 : 0) | (2 * na <= nb ? 2 : 0) | (uneven(ph) ? 4 : 0)));
+        ratio.push_back(static_cast<char>((2 * nb <= na ? 1 : 0) | (2 * na <= nb ? 2 : 0) | (uneven(ph) ? 4 : 0) |
+                                          (blocks_pow2(ph) ? 8 : 0)));
     }
     const bool many = all >= 3000000;
     struct Sums {  // elements by what their tiles are
         int64_t poor = 0, mis = 0, runs = 0, boxes = 0, small = 0, src_mis = 0, part = 0, neat = 0, coarse = 0, fine = 0,
-                trans = 0, odd16 = 0, wide = 0;
+                trans = 0, odd16 = 0, wide = 0, whole = 0;
     };
     auto count = [&](const TileDesc &d, Sums &c) {
         const int64_t e = static_cast<int64_t>(d.nx) * d.ny;
@@ -500,6 +517,7 @@ uint32_t take_patches(const Plan &plan, std::vector<TileDesc> &list, PatchList &
         const int r = ratio[d.prob];
         if (r & 1) c.coarse += e;
         if (r & 2) c.fine += e;
+        if ((r & 8) && !misaligned && (d.flags & TF_FAST) && d.nx == 32 && d.ny == 32) c.whole += e;
         if (tr) c.trans += e;
         if (tr && static_cast<int64_t>(d.sld) * es % 32768 == 0) c.wide += e;
         if ((r & 4) && tr && (d.flags & TF_FAST) && d.nx >= 16 && d.ny >= 16) c.odd16 += e;
@@ -518,11 +536,11 @@ uint32_t take_patches(const Plan &plan, std::vector<TileDesc> &list, PatchList &
         }
     });
     int64_t poor = 0, mis = 0, runs = 0, boxes = 0, small = 0, src_mis = 0, part = 0, neat = 0, coarse = 0, fine = 0,
-            trans = 0, odd16 = 0, wide = 0;
+            trans = 0, odd16 = 0, wide = 0, whole = 0;
     for (const Sums &c : part_sums) {
         poor += c.poor, mis += c.mis, runs += c.runs, boxes += c.boxes, small += c.small, src_mis += c.src_mis;
         part += c.part, neat += c.neat, coarse += c.coarse, fine += c.fine, trans += c.trans, odd16 += c.odd16;
-        wide += c.wide;
+        wide += c.wide, whole += c.whole;
     }
     const size_t n = plan.probs.size();
     const bool beyond = 8 * all * es > (es == 8 ? 7 : 8) * kL2Bytes;  // B and A: 1.75 or 2 times the L2
@@ -565,6 +583,8 @@ uint32_t take_patches(const Plan &plan, std::vector<TileDesc> &list, PatchList &
     if (es == 16 || !beyond || 2 * runs >= all || 2 * small >= all ||
         2 * src_mis >= all || (es == 4 && 2 * part >= all))
         return 0;
+    const bool copies_only = es == 4 && all < 47000000 && 8 * whole >= 7 * all;
+    if (copies_only && 2 * trans < all) return 0;
     for (size_t k = 0; k < n; ++k)
         if (!append_patches(plan.probs[k], static_cast<int>(k), all, out)) {
             out.patches.clear();
@@ -572,17 +592,18 @@ uint32_t take_patches(const Plan &plan, std::vector<TileDesc> &list, PatchList &
             return 0;
         }
     const bool cut = es == 4 && 4 * trans >= 3 * all && 4 * out.cells.size() > 5 * out.patches.size();
-    if (cut && 2 * coarse >= all && all < 50000000) {
+    const bool copies_stay = cut || (es == 4 && 2 * wide >= all);
+    if (copies_stay && (copies_only || (cut && 2 * coarse >= all && all < 50000000))) {
         out.patches.clear();
         out.cells.clear();
         return 0;
     }
-    const bool copies_stay = cut || (es == 4 && 2 * wide >= all);
-    if (!copies_stay && (es == 4 || cplx || mis > 0)) {
+    if (!copies_stay && !copies_only && (es == 4 || cplx || mis > 0)) {
         list.clear();
         return kAllKinds;
     }
     rest = false;
+    if (copies_only) return kCopies;
     if (copies_stay) return kAllKinds & ~kCopies;
     return kAlignedPatchKinds | (4 * boxes < 3 * all ? 1u << K_AXPBY : 0u);
 }

@@ -106,13 +106,22 @@ def test_lists_of_poor_tiles(dtype, op, mb, ma, m, n, pads, want):
     ("c64", "T", 64, 128, 3840, OF["c64"]),
     ("c128", "T", 64, 128, 6016, NONE),
     ("f32", "T", 64, 128, 5632, NONE),  # twice the L2
-    ("f32", "T", 64, 128, 5760, ALL),
+    ("f32", "T", 64, 128, 5760, {"copy", "scale"}),
+    ("f32", "N", 64, 128, 5760, NONE),
+    ("f32", "T", 64, 128, 6848, {"copy", "scale"}),
+    ("f32", "N", 64, 128, 6848, NONE),
+    ("f32", "T", 64, 128, 6912, ALL),
+    ("f32", "N", 64, 128, 6912, ALL),
     ("f64", "T", 40, 40, 8000, {"copy", "axpby", "axpby2"}),  # TMA could stage too few tiles
     ("f32", "T", 24, 100, 8000, NONE),  # ragged cells
     ("f32", "T", 48, 96, 8064, {"axpby", "axpby2"}),  # cells meet inside most patches
     ("f32", "N", 48, 96, 8064, ALL),
     ("f32", "T", 96, 48, 6144, NONE),  # ... A's blocks the smaller ones
     ("f32", "T", 96, 48, 7104, {"axpby", "axpby2"}),
+    ("f32", "T", 96, 96, 6144, ALL),  # whole tiles, but blocks of no power of two
+    ("f32", "T", 64, 128, 6148, {"copy", "scale"}),
+    ("f32", "T", 64, 128, 6145, ALL),  # ragged
+    ("f32", "N", 64, 128, 6145, ALL),
 ])
 def test_lists_of_full_tiles(dtype, op, mb, ma, m, want):
     assert kinds(dtype, op, mb, ma, m) == want
@@ -177,6 +186,13 @@ def test_f32_columns_32_kb_apart_count_by_their_share():
     A = L.packed_blocks(np.arange(0, 8193, 128), np.arange(0, 8193, 128), np.zeros((64, 64)), 1)
     B = L.packed_blocks([0, 0, 8192], [0, 8192], np.zeros((2, 1)), 1)  # ld 1 of the empty block
     assert dispatch("f32", (A, B, "T"))["patch_kinds"] == {"axpby", "axpby2"}
+
+
+@pytest.mark.parametrize("op", ["N", "T"])
+def test_f32_lists_that_are_a_quarter_misaligned(op):
+    """One rank row in four with an odd leading dimension: every kind moves, at
+    sizes where whole aligned tiles of some kinds stay."""
+    assert kinds("f32", op, 64, 128, 6145, grid=4) == ALL
 
 
 def test_targets_of_whole_runs_stay_on_tiles():
