@@ -236,6 +236,17 @@ bool one_order(const costa_layout_s *L, int &order) {
     return any;
 }
 
+// Whether at least half of a layout's elements lie in blocks whose leading
+// dimension is a multiple of `step`.
+bool mostly_ld_multiple(const costa_layout_s *L, int step) {
+    int64_t sum = 0;
+    for (int i = 0; i < L->nbr; ++i)
+        for (int j = 0; j < L->nbc; ++j)
+            if (L->blocks[static_cast<size_t>(i) * L->nbc + j].ld % step == 0)
+                sum += (L->R[i + 1] - L->R[i]) * (L->C[j + 1] - L->C[j]);
+    return 2 * sum >= L->m * L->n;
+}
+
 }  // namespace
 
 bool append_patches(const ProblemHost &ph, int prob, int64_t total, PatchList &out) {
@@ -287,14 +298,14 @@ bool append_patches(const ProblemHost &ph, int prob, int64_t total, PatchList &o
     //   f32    BC50 -> BC75 T 123 / 108, N 111 / 107, odd lds T 110 / 117, N
     //          114 / 108, BC64 -> BC8 N 197 / 100
     //   c128   BC50 -> BC75 T 190 / 196, N 194 / 188
-    // and not for a transposed source whose columns lie a multiple of 1 KB
+    // and not for a transposed source whose columns lie (mostly) a multiple of 1 KB
     // apart, where fewer rows in flight crowd the same channels: f32 T BC64 ->
     // BC8 131 / 198, BC8 -> BC64 106 / 130, BC16 -> BC48 beta = 0.5 153 / 172.
     const AxisPatches &lane_axis = transpose ? Y : X;
     size_t longest = 0;
     for (size_t cy = 0; cy + 1 < Y.chain0.size(); ++cy) longest = std::max(longest, Y.chain0[cy + 1] - Y.chain0[cy]);
-    const bool aligned_ld = static_cast<int64_t>(B->blocks[0].ld) * es % 1024 == 0;
-    const bool mix = lane_axis.shared * (transpose ? 350 : 1024) > lane_axis.extent * es && !(transpose && aligned_ld);
+    const bool mix = lane_axis.shared * (transpose ? 350 : 1024) > lane_axis.extent * es &&
+                     !(transpose && mostly_ld_multiple(B, 1024 / es));
     const size_t chunk = mix ? 2 : longest;
     std::vector<size_t> live(Y.chain0.size() - 1);  // the chains with rows left, so that the work is one step per row
     for (size_t cy = 0; cy < live.size(); ++cy) live[cy] = cy;

@@ -147,6 +147,26 @@ def test_chunks_of_aligned_f32_runs(op, mb, ma, pad, chunks):
     assert share > 0.5 if chunks else share < 0.25
 
 
+@pytest.mark.parametrize("ld_pad", [0, 8])
+def test_order_with_an_empty_first_block(ld_pad):
+    """The order of the patches follows the leading dimension of the source's
+    blocks, not that of an empty first one: the same patches with and without
+    one, mixed by rows of the chains only where the columns lie off a multiple
+    of 1 KB."""
+    m = n = 1024
+    A = L.block_cyclic(m, n, 8, 8, 2, 2, name="A")
+    B = L.block_cyclic(n, m, 64, 64, 2, 2, ld_pad=ld_pad, name="B")
+    R = np.concatenate([[0], B.rsplit])
+    grow = lambda a: np.concatenate([a[:1], a])
+    E = L.LayoutSpec(n, m, R, B.csplit, grow(B.owner), B.nranks, grow(B.buf), grow(B.off), grow(B.ld), grow(B.order),
+                     B.bufsize, name="B")
+    LA, L1, L2 = _layout(A, "f32"), _layout(B, "f32"), _layout(E, "f32")
+    one, two = costa.costa_debug_patches(LA, L1, "T"), costa.costa_debug_patches(LA, L2, "T")
+    assert np.array_equal(one[0], two[0]) and np.array_equal(one[1], two[1])
+    step = np.diff(one[0]["dst"].astype(np.int64)) >> 32  # changes of the rank's buffer of A
+    assert (np.count_nonzero(step) == 3) == (ld_pad == 0)
+
+
 def test_planning_time_of_one_long_chain_beside_many_short_ones():
     """The order that mixes the chains' rows takes one step per row of
     patches: a target of one wide block beside 60,000 single columns, over
