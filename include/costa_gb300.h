@@ -577,8 +577,11 @@ costa_status costa_debug_patches(costa_layout A, costa_layout B, costa_op op, vo
  * when they are the same problems' for the kinds that do not run on patches,
  * then the tiles, the misaligned tiles, the small pieces, the x-halves (cut
  * into more where a list is short), and the kinds whose tiles and whose
- * x-halves TMA may stage.  ops: host, n values. */
-costa_status costa_debug_dispatch(int n, const costa_layout *A, const costa_layout *B, const costa_op *ops,
+ * x-halves TMA may stage.  The choice depends on where the storage lies: host =
+ * 0 on the device, 1 A's, 2 B's, 3 both in host memory, -1 as the last plan of
+ * the layouts found it (on the device before the first).  ops: host array of n
+ * values. */
+costa_status costa_debug_dispatch(int n, const costa_layout *A, const costa_layout *B, const costa_op *ops, int host,
                                   int64_t *out);
 
 /* Diagnostics: TMA staging of the tile kernel's source tiles.  By default

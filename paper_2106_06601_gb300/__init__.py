@@ -89,7 +89,7 @@ def _load():
         "costa_debug_split": [P, P, I, P, I64, P, I64, P, I64, P, P, P],
         "costa_debug_halves": [P, P, I, P, I64, P],
         "costa_debug_patches": [P, P, I, P, I64, P, I64, P, P],
-        "costa_debug_dispatch": [I, P, P, P, P],
+        "costa_debug_dispatch": [I, P, P, P, I, P],
         "costa_debug_groups": [P, P, I, I, P, I64, P],
         "costa_phase_timing": [I],
         "costa_phase_times": [P, P],
@@ -652,16 +652,18 @@ def costa_debug_patches(A: Layout, B: Layout, op: str):
 KINDS = ("copy", "scale", "axpby", "cplx", "axpby2", "cscale", "cplxr")  # the combine kinds, by bit
 
 
-def costa_debug_dispatch(As, Bs, ops) -> dict:
+def costa_debug_dispatch(As, Bs, ops, host: int = -1) -> dict:
     """The work lists that direct calls of a batch run: the kinds that run on
-    patches or may be staged by TMA as sets of names, and the lists' sizes."""
+    patches or may be staged by TMA as sets of names, and the lists' sizes.
+    `host`: 1 A, 2 B has storage in host memory (-1: as the last plan of these
+    layouts found it)."""
     n = len(As)
     ha = (ctypes.c_void_p * n)(*[a.handle.value for a in As])
     hb = (ctypes.c_void_p * n)(*[b.handle.value for b in Bs])
     op = _i32([OPS[o] for o in ops])
     assert op.size == n
     out = np.zeros(10, np.int64)
-    _check(_lib.costa_debug_dispatch(n, ha, hb, _p(op), _p(out)))
+    _check(_lib.costa_debug_dispatch(n, ha, hb, _p(op), host, _p(out)))
     kinds = lambda bits: {k for i, k in enumerate(KINDS) if (int(bits) >> i) & 1}
     return {"patch_kinds": kinds(out[0]), "patches": int(out[1]), "cells": int(out[2]), "tiles_are_rest": bool(out[3]),
             "tiles": int(out[4]), "misaligned": int(out[5]), "pieces": int(out[6]), "halves": int(out[7]),

@@ -261,7 +261,8 @@ PointerAttrFn pointer_attr_fn() {
 }
 
 struct AccessRange {
-    uint64_t lo, hi;  // [lo, hi)
+    uint64_t lo, hi;    // [lo, hi)
+    bool host = false;  // host memory
 };
 
 // The allocation holding `p` if the device `dev` may access it; on failure
@@ -287,6 +288,7 @@ bool access_range(uint64_t p, int dev, AccessRange &r, std::string &why) {
             why = "host memory not mapped at the same address on the device";
             return false;
         }
+        r.host = true;
         break;
     default:
         why = "pageable host memory (allocate it with cudaHostAlloc or register it with cudaHostRegister)";
@@ -311,6 +313,7 @@ bool access_range(uint64_t p, int dev, AccessRange &r, std::string &why) {
 // checked (the multi-GPU exchange), and the result is not cached.
 costa_status check_access_impl(costa_layout_s *L, int dev, const char *which, const int *place, int g) {
     if (!place && L->checked_device == dev) return COSTA_OK;
+    if (!place) L->on_host = false;
     const int64_t es = esize_of(L->dt);
     std::vector<AccessRange> known;  // sorted by lo, disjoint
     auto covered = [&](uint64_t a, uint64_t b) {  // [a, b] inside one known range
@@ -343,6 +346,7 @@ costa_status check_access_impl(costa_layout_s *L, int dev, const char *which, co
             std::string why;
             if (!access_range(first, dev, r, why))
                 return fail(COSTA_ERR_LAYOUT, "%s block (%d, %d): %s", which, i, j, why.c_str());
+            if (!place) L->on_host |= r.host;
             if (r.hi <= end) {  // no range from the driver, or the block leaves it
                 AccessRange r2;
                 if (!access_range(end, dev, r2, why))
@@ -394,14 +398,13 @@ costa_status check_access(costa_layout_s *L, int dev, const char *which) {
 //                  -> 139; c128 beta = 0.5 375 -> 266
 // f32 with only B's ld odd: copy 99 -> 105 (kept on the window path).
 // Doubles in aligned cells whose extents are powers of two from 8 on keep the
-// kinds that read A on the tile kernels in lists of middle size, where a
-// patch kernel's two or three rounds of patches leave the last one half empty
-// (T, us, tiles / patches): beta = 0.5 BC8 1536^2 15.4 / 12.6, 1664^2 16.8 /
+// kinds that read A on the tile kernels in lists of middle size (the lines, here
+// and below, are sizes measured on 152 SMs, in elements; T, us, tiles / patches): beta = 0.5 BC8 1536^2 15.4 / 12.6, 1664^2 16.8 /
 // 17.1, 2816^2 35.3 / 36.9, BC16 -> BC32 4096^2 66.7 / 68.8, 5120^2 faster;
 // beta = 0.7 BC8 -> BC64 2048^2 25.3 / 26.6, 6144^2 154.9 / 162.6.  With op's
 // runs along A's and B's blocks the larger ones, lines of B are shared and the
-// line lies lower (BC64 -> BC8, N, beta = 0.5: 2816^2 37.9 / 38.5, 4096^2 1.23
-// times faster).  alpha = 1.5 with blocks of different sizes likewise (BC8 ->
+// line lies lower (BC64 -> BC8, N, beta = 0.5, 2 x 2 grid: 2816^2 37.9 / 37.5, 4096^2
+// 81 / 67; on 4 x 4, where fewer are shared, 67 / 69, beta = 0.7 74 / 79).  alpha = 1.5 with blocks of different sizes likewise (BC8 ->
 // BC64 2048^2 faster, 4096^2 50.2 / 52.4, 6144^2 104.7 / 108.0).  8-byte copies
 // of partial but not small tiles stay up to 1.75 times the L2 (BC48 2048^2 13.4
 // / 14.2, 2816^2 23.3 / 23.9, BC24 3072^2 26.6 / 27.5, BC48 4096^2 48.0 / 44.7),
@@ -441,13 +444,38 @@ costa_status check_access(costa_layout_s *L, int dev, const char *which) {
 // 1.01, 7040^2 0.97, 1.00, 0.96; N 1.04, 1.03, 1.01, 1.03, 1.03, 0.99, 1.02, 1.02,
 // 0.96; N copy 1.02, 1.01, 1.00, 1.01, 1.01, 0.99, 1.00, 1.01, 0.98.  (BC96 -> BC96
 // 0.91 to 1.00 all over; ragged 6001 x 6003 T beta = 0.5 0.93, N copy 0.87.)  c128 copy (16384^2) 1321 -> 1329 stays on the tiles.
+//
+// Storage in host memory (of any block) that the kernels reach over the host
+// link: patches win there too where their longer writes or the alignment count,
+// but their reads are shorter than a tile's, and over the link that costs more
+// than it does from DRAM.  Tiles / patches, us per call, f64, f32 4096^2, c128
+// 2880^2 unless noted:
+//   c128  B on the host: copy BC8 T 691 / 1105, N 652 / 1101, BC50 -> BC75 T 870 /
+//         1160; both there: BC8 T 1049 / 1183, beta = 0.5 1479 / 1787; only A: BC8
+//         beta = 0.5 1.15 times faster, BC50 -> BC75 copy 790 / 860
+//   f32   op N, both there: 8064^2 BC64 -> BC128 copy 1925 / 2294, beta = 0.5 3183 /
+//         3486, BC8 4096^2 1.27 times faster, BC50 -> BC75 1.18 times; only B: 8064^2
+//         1320 / 2146, BC8 474 / 563, BC50 -> BC75 478 / 494, odd lds 397 / 416
+//         T, only B: BC50 -> BC75 494 / 545, but aligned BC8 1.25 times faster; T,
+//         both there, and only A there, T and N: equal to 1.8 times faster (odd
+//         lds T beta = 0.5 3760 / 3865)
+//         (64 matrices of 2048 x 3072, half of them N, both there: 5.43 ms / 5.83 ms)
+//   f64   only B on the host, T, beta = 0.5 BC50 -> BC75 787 / 837, copy 1.4 times
+//         faster; c64 and the other cases: equal to 1.6 times faster
+// So c128 stays on tiles with B there, and otherwise unless most of its tiles are
+// small; f32 with B there, except lists mostly transposed and aligned, and with
+// both sides there also N of small or misaligned tiles and all of T; and the kinds
+// that read A of 8-byte lists that are transposed and misaligned, with B alone
+// there.
+//
 // Returns the kinds that run on patches (bit per kind; 0: no patches).
 // `rest`: the tiles left in `list` are other problems' than the patches'
 // (reason 1), not the same problems' for the other kinds.
 constexpr uint32_t kAllKinds = (1u << K_NKINDS) - 1u;
 constexpr uint32_t kCopies = (1u << K_COPY) | (1u << K_SCALE);
+constexpr uint32_t kReadsA = (1u << K_AXPBY) | (1u << K_AXPBY2) | (1u << K_CPLX) | (1u << K_CPLXR);
 constexpr uint32_t kAlignedPatchKinds = (1u << K_COPY) | (1u << K_AXPBY2);  // f64; c64: all
-constexpr int64_t kL2Bytes = int64_t(126) << 20;
+constexpr int64_t kL2Bytes = int64_t(126) << 20;  // near GB300's 129 MiB; the lines below were measured with it
 
 // The longest block along one axis (a submatrix starts and ends with parts of
 // blocks).
@@ -478,7 +506,8 @@ bool uneven(const ProblemHost &ph) {
     return odd(block_extent(A.R), block_extent(t ? B.C : B.R)) || odd(block_extent(A.C), block_extent(t ? B.R : B.C));
 }
 
-uint32_t take_patches(const Plan &plan, std::vector<TileDesc> &list, PatchList &out, bool &rest) {
+// `host`: 1 A, 2 B has storage in host memory.
+uint32_t take_patches(const Plan &plan, int host, std::vector<TileDesc> &list, PatchList &out, bool &rest) {
     rest = true;
     if (list.empty() || tma_mode() == 1) return 0;  // COSTA_TMA=1: every kind through the TMA tiles
     const int es = plan.esize;
@@ -542,6 +571,12 @@ uint32_t take_patches(const Plan &plan, std::vector<TileDesc> &list, PatchList &
         part += c.part, neat += c.neat, coarse += c.coarse, fine += c.fine, trans += c.trans, odd16 += c.odd16;
         wide += c.wide, whole += c.whole;
     }
+    const bool odd = 20 * mis >= all;  // a twentieth of the list or more is misaligned
+    if (es == 16 && ((host & 2) || (host && 2 * small < all))) return 0;
+    if (es == 4 && (host & 2)) {
+        const bool across = 4 * trans >= 3 * all;
+        if (across ? host == 2 && odd : host == 2 || (!odd && 2 * small < all)) return 0;
+    }
     const size_t n = plan.probs.size();
     const bool beyond = 8 * all * es > (es == 8 ? 7 : 8) * kL2Bytes;  // B and A: 1.75 or 2 times the L2
     if (2 * poor >= all || (es == 8 && 20 * mis >= all)) {
@@ -565,6 +600,9 @@ uint32_t take_patches(const Plan &plan, std::vector<TileDesc> &list, PatchList &
         if (es == 4 && mis == 0 && 4 * odd16 >= 3 * all && all >= 2400000 &&
             std::find(taken.begin(), taken.end(), 0) == taken.end())
             stay = 2 * coarse >= all ? kAllKinds : kCopies;
+        if (es == 8 && host == 2 && odd && 2 * trans >= all &&
+            std::find(taken.begin(), taken.end(), 0) == taken.end())
+            stay |= kReadsA;
         if (stay == kAllKinds) {
             out.patches.clear();
             out.cells.clear();
@@ -583,7 +621,7 @@ uint32_t take_patches(const Plan &plan, std::vector<TileDesc> &list, PatchList &
     if (es == 16 || !beyond || 2 * runs >= all || 2 * small >= all ||
         2 * src_mis >= all || (es == 4 && 2 * part >= all))
         return 0;
-    const bool copies_only = es == 4 && all < 47000000 && 8 * whole >= 7 * all;
+    const bool copies_only = es == 4 && host == 0 && all < 47000000 && 8 * whole >= 7 * all;
     if (copies_only && 2 * trans < all) return 0;
     for (size_t k = 0; k < n; ++k)
         if (!append_patches(plan.probs[k], static_cast<int>(k), all, out)) {
@@ -629,8 +667,15 @@ struct DirectLists {
     uint32_t tma_big = 0, tma_halves = 0;  // the kinds whose tiles TMA may stage
 };
 
+// Where storage lies in host memory, as check_access found it: 1 A, 2 B.
+int host_storage(const Plan &plan) {
+    int host = 0;
+    for (const ProblemHost &ph : plan.probs) host |= (ph.A->on_host ? 1 : 0) | (ph.B->on_host ? 2 : 0);
+    return host;
+}
+
 // Cuts the plan's problems into the lists that its direct calls run.
-costa_status direct_lists(const Plan &plan, DirectLists &out) {
+costa_status direct_lists(const Plan &plan, int host, DirectLists &out) {
     const int n = static_cast<int>(plan.probs.size()), es = plan.esize, ts = plan.ts;
     // the direct tile list, in (problem, row piece, column piece) order
     std::vector<TileDesc> list;
@@ -654,7 +699,7 @@ costa_status direct_lists(const Plan &plan, DirectLists &out) {
     const costa_status st = check_extents(list, es, "direct");
     if (st != COSTA_OK) return st;
     const bool cplx = plan.dtype == COSTA_C64 || plan.dtype == COSTA_C128;
-    out.patch_kinds = take_patches(plan, list, out.patches, out.rest);
+    out.patch_kinds = take_patches(plan, host, list, out.patches, out.rest);
     if (n == 1) order_direct_tiles(plan.probs[0], list, 0, es, ts);
     out.split = split_small(std::move(list), es, cplx);
     // The aligned tiles also as x-halves (see use_halves), for the kinds
@@ -714,7 +759,7 @@ costa_status build_plan(int n, const costa_layout *As, const costa_layout *Bs, c
         plan->probs.push_back(std::move(ph));
     }
     DirectLists lists;
-    costa_status st = direct_lists(*plan, lists);
+    costa_status st = direct_lists(*plan, host_storage(*plan), lists);
     if (st != COSTA_OK) return st;
     const SplitList &split = lists.split;
     const std::vector<TileDesc> &halves = lists.halves;
@@ -1767,9 +1812,9 @@ costa_status costa_debug_patches(costa_layout A, costa_layout B, costa_op op, vo
     return COSTA_OK;
 }
 
-costa_status costa_debug_dispatch(int n, const costa_layout *A, const costa_layout *B, const costa_op *ops,
+costa_status costa_debug_dispatch(int n, const costa_layout *A, const costa_layout *B, const costa_op *ops, int host,
                                   int64_t *out) {
-    if (n < 1 || n > 65535 || !A || !B || !ops || !out) return fail(COSTA_ERR_INVALID_ARG, "bad arguments");
+    if (n < 1 || n > 65535 || host < -1 || host > 3 || !A || !B || !ops || !out) return fail(COSTA_ERR_INVALID_ARG, "bad arguments");
     Plan plan;
     for (int k = 0; k < n; ++k) {
         costa_status s = validate_pair(A[k], B[k], ops[k]);
@@ -1781,7 +1826,11 @@ costa_status costa_debug_dispatch(int n, const costa_layout *A, const costa_layo
     plan.ts = tile_extent(plan.esize);
     for (int k = 0; k < n; ++k) plan.probs.push_back(make_problem(A[k], B[k], ops[k], plan.ts));
     DirectLists l;
-    const costa_status s = direct_lists(plan, l);
+    if (host < 0) {
+        std::lock_guard<std::mutex> lock(g_mu);  // a plan under construction may be looking at the storage
+        host = host_storage(plan);
+    }
+    const costa_status s = direct_lists(plan, host, l);
     if (s != COSTA_OK) return s;
     const int64_t v[10] = {l.patch_kinds, static_cast<int64_t>(l.patches.patches.size()),
                            static_cast<int64_t>(l.patches.cells.size()), l.rest ? 1 : 0,

@@ -38,6 +38,7 @@ struct costa_layout_s {
     std::vector<int32_t> owner;
     std::vector<costa::DevBlock> blocks;
     int checked_device = -1;  // device whose access to every block was checked
+    bool on_host = false;     // the check found storage in host memory
 };
 
 namespace costa {

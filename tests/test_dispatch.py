@@ -30,11 +30,11 @@ def _pair(dtype, op, mb, ma, m, n, pads=(0, 0), grid=2):
     return A, B
 
 
-def dispatch(dtype, *problems):
+def dispatch(dtype, *problems, host=-1):
     """costa_debug_dispatch of (A, B, op) specs, the kinds those of the type."""
     As, Bs = [_layout(A, dtype) for A, _, _ in problems], [_layout(B, dtype) for _, B, _ in problems]
     try:
-        d = costa.costa_debug_dispatch(As, Bs, [op for _, _, op in problems])
+        d = costa.costa_debug_dispatch(As, Bs, [op for _, _, op in problems], host)
     finally:
         for x in As + Bs:
             x.destroy()
@@ -51,9 +51,9 @@ def dispatch(dtype, *problems):
     return d
 
 
-def kinds(dtype, op, mb, ma, m, n=None, pads=(0, 0), grid=2):
+def kinds(dtype, op, mb, ma, m, n=None, pads=(0, 0), grid=2, host=-1):
     A, B = _pair(dtype, op, mb, ma, m, n or m, pads, grid)
-    return dispatch(dtype, (A, B, op))["patch_kinds"]
+    return dispatch(dtype, (A, B, op), host=host)["patch_kinds"]
 
 
 ALL, NONE = REAL, set()
@@ -186,6 +186,29 @@ def test_f32_columns_32_kb_apart_count_by_their_share():
     A = L.packed_blocks(np.arange(0, 8193, 128), np.arange(0, 8193, 128), np.zeros((64, 64)), 1)
     B = L.packed_blocks([0, 0, 8192], [0, 8192], np.zeros((2, 1)), 1)  # ld 1 of the empty block
     assert dispatch("f32", (A, B, "T"))["patch_kinds"] == {"axpby", "axpby2"}
+
+
+@pytest.mark.parametrize("dtype, op, mb, ma, m, pads, device, a_host, b_host, both", [
+    ("c128", "T", 8, 8, 600, (0, 0), True, True, False, False),
+    ("c128", "N", 50, 75, 600, (0, 0), True, False, False, False),
+    ("f32", "T", 8, 8, 1000, (0, 0), True, True, True, True),
+    ("f32", "N", 8, 8, 1000, (0, 0), True, True, False, True),
+    ("f32", "T", 50, 75, 1000, (0, 0), True, True, False, True),
+    ("f32", "N", 50, 75, 1000, (0, 0), True, True, False, True),
+    ("f32", "N", 64, 128, 1024, (1, 1), True, True, False, True),
+    ("f32", "T", 64, 128, 8064, (0, 0), True, True, True, True),
+    ("f32", "N", 64, 128, 8064, (0, 0), True, True, False, False),
+    ("f64", "T", 50, 75, 1000, (0, 0), True, True, {"copy", "scale"}, True),
+    ("f64", "N", 50, 75, 1000, (0, 0), True, True, True, True),
+    ("c64", "T", 50, 75, 1000, (0, 0), True, True, {"copy", "scale", "cscale"}, True),
+    ("f64", "T", 64, 128, 3840, (0, 0), {"copy", "axpby2"}, {"copy", "axpby2"}, {"copy", "axpby2"}, {"copy", "axpby2"}),
+])
+def test_storage_in_host_memory(dtype, op, mb, ma, m, pads, device, a_host, b_host, both):
+    """Where B's storage is in host memory, lists whose patches would read it in
+    shorter pieces than tiles do stay on tiles."""
+    for host, want in enumerate((device, a_host, b_host, both)):
+        want = OF[dtype] if want is True else want or NONE
+        assert kinds(dtype, op, mb, ma, m, pads=pads, host=host) == want, host
 
 
 @pytest.mark.parametrize("op", ["N", "T"])

@@ -61,6 +61,43 @@ def test_pinned_host_storage_matches_oracle(case, mode, dev):
         LB.destroy()
 
 
+@pytest.mark.parametrize("dtype, op, mb, ma", [("c128", "T", 8, 8), ("c128", "N", 50, 75), ("f32", "N", 8, 8), ("f32", "T", 50, 75),
+                                               ("f64", "T", 50, 75), ("c64", "N", 8, 16)])
+@pytest.mark.parametrize("a_host, b_host", [(True, True), (True, False), (False, True)])
+def test_work_lists_follow_where_the_storage_lies(dtype, op, mb, ma, a_host, b_host, dev):
+    """The planner sees which side is in host memory and chooses the work lists
+    for it; the results equal the oracle's on either, as they do on the device."""
+    import oracle
+    from workloads import layouts as L
+    from workloads.materialize import DeviceMatrix
+    m, n = 150, 203
+    B = L.block_cyclic(*((m, n) if op == "N" else (n, m)), mb, mb, 2, 2, name="B")
+    A = L.block_cyclic(m, n, ma, ma, 2, 2, grid_order="C", name="A")
+    for alpha, beta in ((1.0, 0.0), (2.0, 0.5)):
+        hb = HostMatrix(B, dtype).fill("uniform", C.SEED0 + 19, lambda r: r)
+        ha = HostMatrix(A, dtype).fill("uniform", C.SEED0 + 20, lambda r: r)
+        want = ha.copy()
+        oracle.transform(dtype, op, alpha, beta, A, want.buffers(), B, hb.buffers())
+        place = []
+        for spec, h, on_host in ((A, ha, a_host), (B, hb, b_host)):
+            t = _pinned(h) if on_host else DeviceMatrix(spec, dtype, dev).upload(h)
+            ptrs = _ptrs(spec, h, t) if on_host else t.block_ptrs()
+            place.append((t, costa.costa_layout_from_spec(spec, dtype, ptrs)))
+        (At, LA), (_, LB) = place
+        before = costa.costa_debug_dispatch([LA], [LB], [op])
+        costa.costa_transform(LA, LB, op, alpha, beta, stream=torch.cuda.current_stream(dev).cuda_stream)
+        torch.cuda.synchronize(dev)
+        got = At.numpy() if a_host else At.download().arena
+        assert np.array_equal(got, want.arena)
+        assert before == costa.costa_debug_dispatch([LA], [LB], [op], host=0)  # not looked at yet
+        lists = costa.costa_debug_dispatch([LA], [LB], [op], host=(1 if a_host else 0) | (2 if b_host else 0))
+        assert costa.costa_debug_dispatch([LA], [LB], [op]) == lists
+        if dtype == "c128" and b_host:
+            assert not lists["patch_kinds"] and before["patch_kinds"]
+        LA.destroy()
+        LB.destroy()
+
+
 def test_pageable_host_storage_is_rejected(dev):
     from workloads.materialize import DeviceMatrix
     p = C.fuzz_problem(3)
