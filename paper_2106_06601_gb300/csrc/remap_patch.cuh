@@ -6,7 +6,9 @@
 // What bounds the tile kernel there: a tile lies in one overlay cell, so
 // small or odd cells leave lanes idle, bytes out of flight and a descriptor
 // per few hundred bytes.  A patch (patches.cpp) is a window of A's storage
-// instead, over as many cells as it takes: always about 32 x 32 elements, its
+// instead, over as many cells as it takes: 32 x 32 elements (16 x 16 of 16
+// bytes; a half or a quarter of that in small problems; less at the ends of a
+// rank's local matrix and where more than 8 segments meet along an axis), its
 // writes whole runs of A whatever the blocks.  One warp moves one patch:
 //   1. the patch's cells (source address and stride of each segment pair,
 //      loaded one patch ahead) go to shared memory;
@@ -223,7 +225,9 @@ __device__ __forceinline__ void patch_stage(const PatchDesc &d, const uint4 *cel
 // instruction is issued).  GB300, 8192^2, none / every fourth / every other /
 // all of them on the integer pipes, us per call: f64 T beta = 0.7 BC50 -> BC75
 // 293 / 294 / 287 / 294, odd lds 295 / 295 / 287 / 288, T alpha = 1.5 BC50 ->
-// BC75 206 / 187 / 192 / 240.  c128 (half the values per row) loses 5%.
+// BC75 206 / 187 / 192 / 240.  One share serves both kinds: every other, the
+// best for beta; alpha alone would be 2.6% faster there with every fourth.  c128
+// (half the values per row) loses 5%.
 template <typename T, int N>
 __device__ __forceinline__ void mul_group(Chunk<T> (&v)[N], double c, unsigned mask) {
     double *d = reinterpret_cast<double *>(v);

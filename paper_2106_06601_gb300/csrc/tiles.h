@@ -120,8 +120,8 @@ void append_direct_tiles(const ProblemHost &ph, int prob, int es, int ts, std::v
 
 // A list of few tiles with each tile cut into 2 or 4 by rows of its target
 // (multiples of 4 rows), so that more warps share it: at most few_tiles tiles
-// result (the tile kernel runs at least that many warps).  GB300, T copy, us
-// per call: f64 128^2 2.8 -> 1.9, 512^2 2.9 -> 2.1, 1024^2 3.3 -> 3.1; f32 256^2
+// result (the tile kernel runs at least that many warps: 4 or 16 on each of 152
+// SMs).  GB300, T copy, us per call: f64 128^2 2.8 -> 1.9, 512^2 2.9 -> 2.1, 1024^2 3.3 -> 3.1; f32 256^2
 // 2.1 -> 1.8; c128 256^2 3.8 -> 2.2, 512^2 3.9 -> 2.9.
 inline size_t few_tiles(int es) { return es == 16 ? 608 : 2432; }
 std::vector<TileDesc> cut_few(std::vector<TileDesc> &&list, int es);
