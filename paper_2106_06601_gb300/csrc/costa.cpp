@@ -413,6 +413,22 @@ costa_status check_access(costa_layout_s *L, int dev, const char *which) {
 // faster), with A's blocks the smaller ones every kind (BC48 -> BC16 8192^2
 // beta = 0.5 142 / 144).
 //
+// Blocks stored apart: where the blocks of a rank do not continue each other in
+// storage (tiles stored one by one, in any order), a patch ends with its block,
+// and a warp that moves 8 x 8 elements has little in flight.  A problem keeps
+// its tiles if its patches are many and hold fewer than 300 elements on average
+// (256 below 5 million elements, 100 below 1.2; 16-byte ones 90, 60 below 2.4),
+// unless they are 4.5 (16-byte: 3) times as large as its tiles, or no more than
+// the warps take in about one round (3000; 16-byte ones, which gain longest,
+// 20000).  A stored block by block, B BC64 on 4 x 4, patches / tiles (time, mean of
+// N, T, copy and beta = 0.5; "rows": ranks' blocks side by side in storage):
+//   f64   8 x 8 256^2 0.48, 560^2 0.97, 1536^2 2.2, 4608^2 3.9; 16 x 16 704^2 0.86, 2048^2
+//         0.89, 4608^2 1.17; 8 x 8 rows 1536^2 0.90, 4608^2 1.40;
+//         6 x 6 rows 2048^2 0.77; 4 x 4 rows 3072^2 0.77
+//   f32   8 x 8 256^2 0.60, 1536^2 2.1, 4608^2 3.8; 16 x 16 704^2 0.90, 2048^2 1.03, 4608^2
+//         1.28; 8 x 8 rows 1536^2 0.86, 4608^2 1.24; 6 x 6 rows 0.32
+//   c128  4 x 4 400^2 0.64, 2048^2 2.9; 8 x 8 1536^2 0.93, 3072^2 1.37; 10 x 10 3072^2 0.80
+//
 // 2. Lists of full tiles of 4- and 8-byte elements with 1.75 times (f32: twice)
 // the data that the L2 cache holds and targets that are not one contiguous run per
 // tile: every kind, or for f64 the kinds in kAlignedPatchKinds, run on patches
@@ -579,11 +595,20 @@ uint32_t take_patches(const Plan &plan, int host, std::vector<TileDesc> &list, P
     }
     const size_t n = plan.probs.size();
     const bool beyond = 8 * all * es > (es == 8 ? 7 : 8) * kL2Bytes;  // B and A: 1.75 or 2 times the L2
+    // the most patches of a problem (see "Blocks stored apart" above)
+    auto most = [&](const ProblemHost &ph) {
+        const int64_t e = ph.A->m * ph.A->n,
+                      tiles = static_cast<int64_t>(ph.rows.tiles.size()) * static_cast<int64_t>(ph.cols.tiles.size());
+        const int64_t few = es == 16 ? 20000 : 3000;
+        const int64_t least = es == 16 ? (all < 2400000 ? 60 : 90) : all < 1200000 ? 100 : all < 5000000 ? 256 : 300;
+        const double share = static_cast<double>(e) / static_cast<double>(std::max<int64_t>(all, 1));
+        return std::max({static_cast<int64_t>(share * few), e / least, es == 16 ? tiles / 3 : 2 * tiles / 9});
+    };
     if (2 * poor >= all || (es == 8 && 20 * mis >= all)) {
         std::vector<char> taken(n, 0);
         bool any = false;
         for (size_t k = 0; k < n; ++k)
-            any |= (taken[k] = append_patches(plan.probs[k], static_cast<int>(k), all, out)) != 0;
+            any |= (taken[k] = append_patches(plan.probs[k], static_cast<int>(k), all, most(plan.probs[k]), out)) != 0;
         if (!any) return 0;
         uint32_t stay = 0;
         if (es == 8 && mis == 0 && all >= 2400000 && std::find(taken.begin(), taken.end(), 0) == taken.end()) {
@@ -624,7 +649,7 @@ uint32_t take_patches(const Plan &plan, int host, std::vector<TileDesc> &list, P
     const bool copies_only = es == 4 && host == 0 && all < 47000000 && 8 * whole >= 7 * all;
     if (copies_only && 2 * trans < all) return 0;
     for (size_t k = 0; k < n; ++k)
-        if (!append_patches(plan.probs[k], static_cast<int>(k), all, out)) {
+        if (!append_patches(plan.probs[k], static_cast<int>(k), all, INT64_MAX, out)) {
             out.patches.clear();
             out.cells.clear();
             return 0;
@@ -1802,7 +1827,7 @@ costa_status costa_debug_patches(costa_layout A, costa_layout B, costa_op op, vo
     ph.B = B;
     ph.op = op;
     PatchList l;
-    append_patches(ph, 0, A->m * A->n, l);
+    append_patches(ph, 0, A->m * A->n, INT64_MAX, l);
     *npatches = static_cast<int64_t>(l.patches.size());
     *ncells = static_cast<int64_t>(l.cells.size());
     const size_t kp = static_cast<size_t>(std::min<int64_t>(cap_patches, *npatches));

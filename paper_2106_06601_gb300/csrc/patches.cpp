@@ -249,7 +249,7 @@ bool mostly_ld_multiple(const costa_layout_s *L, int step) {
 
 }  // namespace
 
-bool append_patches(const ProblemHost &ph, int prob, int64_t total, PatchList &out) {
+bool append_patches(const ProblemHost &ph, int prob, int64_t total, int64_t most, PatchList &out) {
     const costa_layout_s *A = ph.A, *B = ph.B;
     int oa = 0, ob = 0;
     if (!one_order(A, oa) || !one_order(B, ob)) return false;
@@ -276,7 +276,7 @@ bool append_patches(const ProblemHost &ph, int prob, int64_t total, PatchList &o
     const AxisPatches &X = a_col ? rows : cols, &Y = a_col ? cols : rows;
     const int64_t ncells = rows.nseg_sum.back() * cols.nseg_sum.back();
     const int64_t npatches = static_cast<int64_t>(X.patches.size()) * static_cast<int64_t>(Y.patches.size());
-    if (static_cast<int64_t>(out.cells.size()) + ncells >= (int64_t(1) << 32)) return false;
+    if (npatches > most || static_cast<int64_t>(out.cells.size()) + ncells >= (int64_t(1) << 32)) return false;
     // Order: per pair of chains (a rank's local matrix) A's storage order, x
     // fastest, so that the patches in flight together form long runs of A.
     struct Row {

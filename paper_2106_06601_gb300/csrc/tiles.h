@@ -149,11 +149,11 @@ bool use_halves(const ProblemHost &ph, int es);
 
 // The patches of problem `prob` (patches.cpp) of a list of `total` elements,
 // appended to `out`; false (and nothing appended) when its layouts mix element
-// orders or need more cells than a patch can index.
+// orders, need more cells than a patch can index, or more than `most` patches.
 struct PatchList {
     std::vector<PatchDesc> patches;
     std::vector<PatchCell> cells;
 };
-bool append_patches(const ProblemHost &ph, int prob, int64_t total, PatchList &out);
+bool append_patches(const ProblemHost &ph, int prob, int64_t total, int64_t most, PatchList &out);
 
 }  // namespace costa

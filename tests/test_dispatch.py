@@ -226,6 +226,33 @@ def test_targets_of_whole_runs_stay_on_tiles():
     assert dispatch("f64", (A, B, "T"))["patch_kinds"] == NONE
 
 
+def _stored_by_block(n, mb, nb, mode):
+    """n x n in mb x nb blocks, each stored on its own: owners at random, or 4 x 4
+    block-cyclic (a rank's blocks of one block row follow each other)."""
+    R, S = np.append(np.arange(0, n, mb), n), np.append(np.arange(0, n, nb), n)
+    i, j = np.meshgrid(np.arange(len(R) - 1), np.arange(len(S) - 1), indexing="ij")
+    own = (i * 7919 + j * 104729 + i * j) % 16 if mode == "rand" else i % 4 * 4 + j % 4
+    return L.packed_blocks(R, S, own, 16)
+
+
+@pytest.mark.parametrize("dtype, n, block, mode, want", [
+    ("f64", 256, (8, 8), "rand", True), ("f64", 704, (8, 8), "rand", False), ("f64", 3072, (8, 8), "rand", False),
+    ("f32", 704, (16, 16), "rand", True), ("f32", 3072, (16, 16), "rand", False),
+    ("f64", 1536, (8, 8), "cyc", True), ("f64", 3072, (8, 8), "cyc", False), ("f32", 3072, (4, 4), "cyc", True),
+    ("f32", 3072, (6, 6), "cyc", True), ("c128", 560, (4, 4), "rand", True), ("c128", 1000, (4, 4), "rand", False),
+    ("c128", 1536, (8, 8), "rand", True), ("c128", 2048, (8, 8), "rand", False), ("c128", 2048, (10, 10), "rand", True),
+])
+def test_blocks_stored_apart(dtype, n, block, mode, want):
+    """Patches end where a rank's blocks do not continue each other in storage:
+    lists of many small ones stay on tiles."""
+    A = _stored_by_block(n, *block, mode)
+    B = L.block_cyclic(n, n, 64, 64, 4, 4, name="B")
+    got = dispatch(dtype, (A, B, "T"))["patch_kinds"]
+    if want and dtype == "f64" and mode == "cyc":
+        got = got | {"axpby", "axpby2"}  # power-of-two cells may keep these
+    assert got == (OF[dtype] if want else NONE)
+
+
 def test_mixed_element_orders_stay_on_tiles():
     """Layouts that mix element orders have no patches; in a batch the other
     problems move to patches, and every kind runs on both lists."""
