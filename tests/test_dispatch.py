@@ -253,6 +253,19 @@ def test_blocks_stored_apart(dtype, n, block, mode, want):
     assert got == (OF[dtype] if want else NONE)
 
 
+@pytest.mark.parametrize("dtype, block, mode, want", [
+    ("f64", 48, "rand", NONE), ("f64", 100, "rand", {"copy", "axpby2"}), ("f64", 48, "cyc", {"copy", "axpby2"}),
+    ("f32", 100, "rand", NONE), ("f32", 48, "cyc", NONE), ("f32", 96, "rand", ALL), ("c64", 48, "rand", NONE),
+    ("c64", 96, "rand", OF["c64"])])
+def test_full_tiles_of_blocks_stored_apart(dtype, block, mode, want):
+    """Lists of full tiles move to patches only where these are nearly whole."""
+    n = 7680
+    A = _stored_by_block(n, block, block, mode)
+    B = L.block_cyclic(n, n, 64, 64, 4, 4, name="B")
+    got = dispatch(dtype, (A, B, "N"))["patch_kinds"]
+    assert got - {"axpby"} == want - {"axpby"}  # (TMA may take the general beta)
+
+
 def test_mixed_element_orders_stay_on_tiles():
     """Layouts that mix element orders have no patches; in a batch the other
     problems move to patches, and every kind runs on both lists."""
